@@ -11,6 +11,8 @@
 // code of their clamped value and are stored exactly in fp16 on the side.
 #include <math.h>
 
+#include <algorithm>
+
 #include "mkv_common.cuh"
 #include "mkv_internal.h"
 #include "mkv_quant_token.cuh"
@@ -142,6 +144,532 @@ __global__ void quantize_kernel(const QuantArgs a) {
                          scr, &g_status_kvquant, [] { __syncthreads(); });
   }
   finish(t_base + a.n_tokens);
+}
+
+// ----------------------------------------------------------------- bulk quantize (a prompt)
+//
+// Many tokens at once: the prompt of every (batch, kv-head) is cut into P * kBulkWarps runs of
+// tokens, one warp each, and a warp quantizes its tokens by itself, without barriers.
+// The CSR of the key outliers needs each run's first entry: quantize_count_kernel counts the runs'
+// outliers (one more pass over the keys), the last CTA of a batch entry turns the counts into entry
+// offsets, and both pass through the CSR slot of the run's first token, which the run overwrites.
+//
+// B = 8, 8 kv-heads, T = 8192, D = 128, 4 bits: 0.32 ms (count 33 us, quantize 287 us), where one CTA
+// per unit with its tokens in order took 13.4 ms (64 CTAs, a barrier chain of ~1.6 us a token).  Bound
+// by instruction issue (about 400 warp instructions a token, IPC 2.5) rather than by its 349 MB, so:
+//  * key codes and outliers are decided on fp16 pairs: for fp16 x, x > mu is x > (mu rounded down),
+//    x < t is x < (t rounded up);
+//  * codebook searches descend a tree of thresholds (ascending midpoints; a codebook out of order is
+//    counted linearly, as quantize_token does): the keys' in registers, the values' upper levels in
+//    registers and their last two in one 16-byte shared-memory read, which keeps 16 warps per SM;
+//  * the n_v largest |x| and the value range of a token are warp reductions (redux.sync) over
+//    order-preserving integer keys;
+//  * a warp takes two tokens at a time, so that their dependent chains overlap (one at a time: 0.50 ms).
+
+constexpr int kBulkWarps = 8;
+constexpr int64_t kBulkMinTokens = 6;
+
+// Token run of warp w of a unit: [w * per_w, (w + 1) * per_w) of the call's n tokens.
+struct BulkSplit {
+  int P;          // CTAs per (batch, kv-head); P * Hkv <= 256 (the tickets in T_len's top 8 bits)
+  int64_t per_w;
+};
+
+// Streaming read of two or four fp16 (volatile: issued where written, so that several are in flight)
+__device__ __forceinline__ uint32_t ld_stream4(const void* p) {
+  uint32_t x;
+  asm volatile("ld.global.nc.L1::no_allocate.u32 %0, [%1];\n" : "=r"(x) : "l"(p));
+  return x;
+}
+__device__ __forceinline__ uint2 ld_stream8(const void* p) {
+  uint2 x;
+  asm volatile("ld.global.nc.L1::no_allocate.v2.u32 {%0, %1}, [%2];\n" : "=r"(x.x), "=r"(x.y) : "l"(p));
+  return x;
+}
+
+template <int D>
+__global__ void __launch_bounds__(kBulkWarps * 32) quantize_count_kernel(const QuantArgs a, const BulkSplit sp) {
+  constexpr int NH = D / 64;               // fp16 pairs per lane
+  const int64_t bh = blockIdx.y;
+  const int b = (int)(bh / a.Hkv), h = (int)(bh % a.Hkv);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  __shared__ int s_last;
+  const int64_t t_base = a.T_len[b] & 0xffffff, n = a.n_tokens;
+  if (t_base + n > a.T_cap) return;        // no room: quantize_bulk_kernel raises the flag
+  __half2 lo[NH], hi[NH];                  // channels NH * 2 * lane ..
+#pragma unroll
+  for (int i = 0; i < NH; ++i) {
+    const int64_t c = (int64_t)h * D + (lane * NH + i) * 2;
+    lo[i] = __halves2half2(__float2half_ru(a.t_lo[c]), __float2half_ru(a.t_lo[c + 1]));
+    hi[i] = __halves2half2(__float2half_rd(a.t_hi[c]), __float2half_rd(a.t_hi[c + 1]));
+  }
+  int32_t* off_row = a.k_out_off + bh * (a.T_cap + 1);
+  const int64_t w0 = ((int64_t)blockIdx.x * kBulkWarps + warp) * sp.per_w, w1 = min(n, w0 + sp.per_w);
+  const int m = (int)max((int64_t)0, w1 - w0);
+  const __half* src = a.k_pre + (bh * n + w0) * D + lane * NH * 2;
+  int cnt = 0;
+  constexpr int U = 8;                     // rows in flight
+  for (int t = 0; t < m; t += U) {
+    uint32_t x[U][NH];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const __half* p = src + (int64_t)min(t + u, m - 1) * D;
+      if constexpr (NH == 2) {
+        const uint2 y = ld_stream8(p);
+        x[u][0] = y.x;
+        x[u][1] = y.y;
+      } else {
+        x[u][0] = ld_stream4(p);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const uint32_t live = t + u < m ? 0x00010001u : 0u;
+#pragma unroll
+      for (int i = 0; i < NH; ++i) {
+        const __half2 v = *reinterpret_cast<const __half2*>(&x[u][i]);
+        cnt += __popc((__hlt2_mask(v, lo[i]) | __hgt2_mask(v, hi[i])) & live);
+      }
+    }
+  }
+  cnt = __reduce_add_sync(0xffffffffu, cnt);
+  if (lane == 0 && w0 < w1) off_row[t_base + w0 + 1] = cnt;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const unsigned old = atomicAdd(reinterpret_cast<unsigned*>(a.T_len) + b, 1u << 24);
+    s_last = (int)(old >> 24) == (int)gridDim.x * a.Hkv - 1;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  for (int hh = warp; hh < a.Hkv; hh += kBulkWarps) {   // counts -> first entries, one warp per kv-head
+    int32_t* row = a.k_out_off + ((int64_t)b * a.Hkv + hh) * (a.T_cap + 1) + t_base;
+    int32_t run = t_base == 0 ? 0 : __ldcg(row);
+    for (int i0 = 0; i0 < sp.P * kBulkWarps; i0 += 32) {
+      const int64_t t = (int64_t)(i0 + lane) * sp.per_w;
+      const bool in = i0 + lane < sp.P * kBulkWarps && t < n;
+      const int32_t c = in ? __ldcg(row + t + 1) : 0;
+      int32_t incl = c;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+      }
+      if (in) row[t + 1] = run + incl - c;
+      run += __shfl_sync(0xffffffffu, incl, 31);
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) a.T_len[b] = (int32_t)t_base;   // the tickets cleared
+}
+
+// #{j : x > m_j} of the 2^BITS - 1 ascending thresholds of a channel: the upper BITS - 2 levels of
+// the search tree in registers (top), then one 16-byte shared-memory read of the three thresholds
+// left, as (middle, lower, upper).  `leaf` is the thread's entry of quadrant 0, STRIDE apart.
+template <int BITS, int STRIDE>
+__device__ __forceinline__ int tree_code(float x, const float (&top)[BITS == 4 ? 3 : 1], const float4* leaf) {
+  int q = 0;
+  if constexpr (BITS == 4) {               // top = m_7, m_3, m_11
+    const bool up = x > top[0];
+    q = (up ? 2 : 0) + (x > (up ? top[2] : top[1]) ? 1 : 0);
+  } else if constexpr (BITS == 3) {        // top = m_3
+    q = x > top[0] ? 1 : 0;
+  }
+  const float4 m = leaf[q * STRIDE];
+  const bool up = x > m.x;
+  return 4 * q + (up ? 2 : 0) + (x > (up ? m.z : m.y) ? 1 : 0);
+}
+// the linear count (any order of the thresholds)
+template <int BITS, int STRIDE>
+__device__ __forceinline__ int count_code(float x, const float (&top)[BITS == 4 ? 3 : 1], const float4* leaf) {
+  int code = 0;
+#pragma unroll
+  for (int q = 0; q < (1 << (BITS - 2)); ++q) {
+    const float4 m = leaf[q * STRIDE];
+    code += (x > m.x) + (x > m.y) + (x > m.z);
+    if (q + 1 < (1 << (BITS - 2))) code += x > top[q];
+  }
+  return code;
+}
+// the same for two fp16 values at once; codes in the two halves
+template <int BITS>
+__device__ __forceinline__ uint32_t tree_code2(__half2 x, const uint32_t (&m)[(1 << BITS) - 1]) {
+  uint32_t cur[(1 << BITS) - 1];
+#pragma unroll
+  for (int i = 0; i < (1 << BITS) - 1; ++i) cur[i] = m[i];
+  uint32_t code = 0;
+#pragma unroll
+  for (int l = BITS - 1; l >= 0; --l) {
+    const int half = (1 << l) - 1;
+    const uint32_t up = __hgt2_mask(x, *reinterpret_cast<const __half2*>(&cur[half]));
+    code |= up & (0x00010001u << l);
+#pragma unroll
+    for (int i = 0; i < half; ++i) cur[i] = (up & cur[half + 1 + i]) | (~up & cur[i]);
+  }
+  return code;
+}
+
+// RN(d / s) for r = RN(1 / s): Markstein's correction (IBM J. Res. Dev. 34, 1990) applied twice, so
+// that the second starts from a faithful quotient.  s is a difference of two fp16 values (or 1/3,
+// 1/7, 1/15 of one) and d one of an fp16 value and such, so no remainder underflows; a quotient
+// beyond 2^30 (d infinite, or far outside the range) is past every code's limit as it is.
+__device__ __forceinline__ float div_rn(float d, float s, float r) {
+  const float q0 = __fmul_rn(d, r);
+  const float q1 = __fmaf_rn(__fmaf_rn(-q0, s, d), r, q0);
+  const float q2 = __fmaf_rn(__fmaf_rn(-q1, s, d), r, q1);
+  return fabsf(q0) < 1073741824.f ? q2 : q0;
+}
+
+__device__ __forceinline__ float f32_from_key(uint32_t k) {
+  return __uint_as_float((k & 0x80000000u) ? k & 0x7fffffffu : ~k);
+}
+
+// A token's code row from the 2 * BITS * (D / 64) bits of each lane's pairs, in lane order.
+template <int D, int BITS>
+__device__ __forceinline__ void store_codes(uint8_t* row, uint32_t x, int lane, bool live) {
+  constexpr int LB = 2 * BITS * (D / 64);
+  if constexpr (LB == 16) {
+    if (live) reinterpret_cast<uint16_t*>(row)[lane] = (uint16_t)x;
+  } else if constexpr (LB == 8) {
+    if (live) row[lane] = (uint8_t)x;
+  } else if constexpr (LB == 4) {
+    const uint32_t y = __shfl_down_sync(0xffffffffu, x, 1);
+    if (live && (lane & 1) == 0) row[lane >> 1] = (uint8_t)(x | (y << 4));
+  } else {                                 // 12 or 6 bits: four lanes fill three 16- or 8-bit units
+    constexpr int S = LB / 3;
+    const uint32_t y = __shfl_down_sync(0xffffffffu, x, 1);
+    const int j = lane & 3, at = (lane >> 2) * 3 + j;
+    const uint32_t w = (x >> (S * j)) | (y << (LB - S * j));
+    if (live && j < 3) {
+      if constexpr (LB == 12)
+        reinterpret_cast<uint16_t*>(row)[at] = (uint16_t)w;
+      else
+        row[at] = (uint8_t)w;
+    }
+  }
+}
+
+template <int D, int BITS, bool NUQ>
+__global__ void __launch_bounds__(kBulkWarps * 32, 2) quantize_bulk_kernel(const QuantArgs a, const BulkSplit sp) {
+  constexpr int NH = D / 64, NC = 2 * NH;  // fp16 pairs and channels per lane
+  constexpr int K = 1 << BITS, L = K - 1, NQ = K / 4, ROW = D * BITS / 8;
+  __shared__ uint32_t s_kmu[NUQ ? NH * L * 32 : 1];   // [pair][threshold][lane] key midpoints rounded down
+  __shared__ float4 s_leaf[NUQ ? NQ * NC * 32 : 1];   // [quadrant][channel][lane] value midpoints
+  const int64_t bh = blockIdx.y;
+  const int b = (int)(bh / a.Hkv), h = (int)(bh % a.Hkv);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t t_base = a.T_len[b] & 0xffffff, n = a.n_tokens;
+  if (t_base + n > a.T_cap) {              // no room: drop, flag, keep T_len
+    if (blockIdx.x == 0 && h == 0 && threadIdx.x == 0) atomicOr(&g_status_kvquant, MKV_FLAG_CACHE_FULL);
+    return;
+  }
+  // channel j of lane l: D = 128: 2 l, 2 l + 1, 64 + 2 l, 65 + 2 l; D = 64: l, 32 + l
+  auto chan_of = [](int j, int l) { return NH == 2 ? 2 * l + (j & 1) + (j >> 1) * 64 : l + j * 32; };
+  auto chan = [&](int j) { return chan_of(j, lane); };
+  bool sorted = true;
+  if constexpr (NUQ) {
+    for (int e = threadIdx.x; e < NC * 32 * L; e += kBulkWarps * 32) {
+      const int j = e / (32 * L), l = e / L % 32, m = e % L;
+      const int64_t hc = ((int64_t)h * D + chan_of(j, l)) * K + m;
+      const float c0 = h2f(a.k_cb[hc]), c1 = h2f(a.k_cb[hc + 1]), v0 = h2f(a.v_cb[hc]), v1 = h2f(a.v_cb[hc + 1]);
+      const float km = fl32_mid(c0, c1), vm = fl32_mid(v0, v1);
+      sorted = sorted && c0 <= c1 && v0 <= v1 && km == km && vm == vm;   // then the midpoints ascend too
+      reinterpret_cast<__half*>(s_kmu)[(((j >> 1) * L + m) * 32 + l) * 2 + (j & 1)] =
+          __float2half_rd(km);
+      // quadrant m / 4 holds m_4q .. m_4q+2 as (middle, lower, upper, the threshold after it)
+      constexpr int at[4] = {1, 0, 2, 3};
+      reinterpret_cast<float*>(s_leaf)[(((m >> 2) * NC + j) * 32 + l) * 4 + at[m & 3]] = vm;
+    }
+  }
+  sorted = __syncthreads_and(sorted);
+  uint32_t lo2[NH], hi2[NH];               // outlier thresholds as fp16 pairs
+  uint32_t kmu[NH][L];
+  float top[NC][BITS == 4 ? 3 : 1];        // the value search's upper levels
+  float klo[NC], ksc[NC];                  // uniform: key grid
+#pragma unroll
+  for (int i = 0; i < NH; ++i) {
+    uint16_t lo[2], hi[2];
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const int j = 2 * i + e;
+      const int64_t hc = (int64_t)h * D + chan(j);
+      lo[e] = __half_as_ushort(__float2half_ru(a.t_lo[hc]));
+      hi[e] = __half_as_ushort(__float2half_rd(a.t_hi[hc]));
+      if constexpr (NUQ) {
+        if constexpr (BITS == 4) {
+          top[j][0] = s_leaf[(1 * NC + j) * 32 + lane].w;
+          top[j][1] = s_leaf[(0 * NC + j) * 32 + lane].w;
+          top[j][2] = s_leaf[(2 * NC + j) * 32 + lane].w;
+        } else {
+          top[j][0] = BITS == 3 ? s_leaf[j * 32 + lane].w : 0.f;
+        }
+      } else {
+        klo[j] = a.k_lo[hc];
+        ksc[j] = a.k_scale[hc];
+      }
+    }
+    lo2[i] = (uint32_t)lo[0] | ((uint32_t)lo[1] << 16);
+    hi2[i] = (uint32_t)hi[0] | ((uint32_t)hi[1] << 16);
+    if constexpr (NUQ) {
+#pragma unroll
+      for (int m = 0; m < L; ++m) kmu[i][m] = s_kmu[(i * L + m) * 32 + lane];
+    }
+  }
+
+  const int64_t w0 = ((int64_t)blockIdx.x * kBulkWarps + warp) * sp.per_w, w1 = min(n, w0 + sp.per_w);
+  int32_t* off_row = a.k_out_off + bh * (a.T_cap + 1) + t_base;
+  if (w0 < w1) {
+    const int m = (int)(w1 - w0);          // this warp's tokens
+    uint32_t* k_out = a.k_out + bh * a.k_out_cap;
+    const int32_t cap = (int32_t)min(a.k_out_cap, (int64_t)INT32_MAX);
+    const int64_t d0 = bh * a.T_cap + t_base + w0;
+    uint32_t* v_out = a.v_out + d0 * a.n_v;
+    float2* v_par = a.v_params + d0;
+    uint8_t* kc = a.k_codes + d0 * ROW;
+    uint8_t* vc = a.v_codes + d0 * ROW;
+    const uint8_t* ks = reinterpret_cast<const uint8_t*>(a.k_pre + (bh * n + w0) * D) + lane * (NH == 2 ? 4 : 2);
+    const uint8_t* vs = reinterpret_cast<const uint8_t*>(a.v + (bh * n + w0) * D) + lane * (NH == 2 ? 4 : 2);
+    const int t0 = (int)((t_base + w0) & 63);
+    off_row += w0 + 1;
+    int32_t off = off_row[0];              // the run's first entry (from quantize_count_kernel)
+    __syncwarp();
+    const unsigned lt = (1u << lane) - 1u;
+    auto load = [&](const uint8_t* base, int t, uint32_t (&x)[NH]) {
+      const uint8_t* p = base + (int64_t)min(t, m - 1) * (D * 2);
+      if constexpr (NH == 2) {
+        x[0] = ld_stream4(p);
+        x[1] = ld_stream4(p + 128);
+      } else {
+        x[0] = (uint32_t)__ldg(reinterpret_cast<const uint16_t*>(p)) |
+               ((uint32_t)__ldg(reinterpret_cast<const uint16_t*>(p + 64)) << 16);
+      }
+    };
+    uint32_t kn[2][NH], vn[2][NH];         // the next two tokens' rows, in flight
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      load(ks, e, kn[e]);
+      load(vs, e, vn[e]);
+    }
+    int32_t my_off = 0;                    // of token 32 * i + lane of the run: end of its entries,
+    float2 my_par = make_float2(0.f, 0.f); // value range
+    // two tokens at a time: their dependent chains (searches, warp reductions, divisions) overlap
+    for (int t = 0; t < m; t += 2) {
+      uint32_t kx[2][NH], vx[2][NH];
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+#pragma unroll
+        for (int i = 0; i < NH; ++i) {
+          kx[e][i] = kn[e][i];
+          vx[e][i] = vn[e][i];
+        }
+        load(ks, t + 2 + e, kn[e]);
+        load(vs, t + 2 + e, vn[e]);
+      }
+      const bool two = t + 1 < m;
+      // a lane's pairs in order: D = 128: (2 lane, 64 + 2 lane), (2 lane + 1, ..); D = 64: (lane, 32 + lane)
+      auto pack = [&](const uint32_t (&c)[NH]) -> uint32_t {
+        if constexpr (NH == 2) {
+          const uint32_t w = c[0] | (c[1] << BITS);
+          return (w & 0xffffu) | ((w >> 16) << (2 * BITS));
+        } else {
+          return (c[0] & 0xffffu) | ((c[0] >> 16) << BITS);
+        }
+      };
+      // ---- values: the n_v largest |x| (ties: lower channel), each found by a warp maximum over
+      // unique keys (|x| as fp16 bits, 255 - channel, sign)
+      uint32_t key[2][NC];
+#pragma unroll
+      for (int e = 0; e < 2; ++e)
+#pragma unroll
+        for (int j = 0; j < NC; ++j) {
+          const uint32_t x = (vx[e][j >> 1] >> (16 * (j & 1))) & 0xffffu;
+          key[e][j] = ((x & 0x7fffu) << 9) | (x >> 15) | (uint32_t)((255 - chan(j)) << 1);
+        }
+#pragma unroll 1
+      for (int r = 0; r < a.n_v; ++r) {
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          uint32_t mx = key[e][0];
+#pragma unroll
+          for (int j = 1; j < NC; ++j) mx = max(mx, key[e][j]);
+          const uint32_t w = __reduce_max_sync(0xffffffffu, mx);
+#pragma unroll
+          for (int j = 0; j < NC; ++j) key[e][j] = key[e][j] == w ? 0u : key[e][j];   // live keys are nonzero
+          if (lane == 0 && (e == 0 || two))
+            v_out[e * a.n_v + r] = ((255u - ((w >> 1) & 255u)) << 16) | (w >> 9) | ((w & 1u) << 15);
+        }
+      }
+      v_out += 2 * a.n_v;
+      // ---- keys: codes (packed by pairs of channels) and outliers
+      uint32_t code[2][NH], om[2][NH];
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+#pragma unroll
+        for (int i = 0; i < NH; ++i) {
+          const __half2 x = *reinterpret_cast<const __half2*>(&kx[e][i]);
+          om[e][i] = __hlt2_mask(x, *reinterpret_cast<const __half2*>(&lo2[i])) |
+                     __hgt2_mask(x, *reinterpret_cast<const __half2*>(&hi2[i]));
+          if constexpr (NUQ) {
+            code[e][i] = tree_code2<BITS>(x, kmu[i]);
+          } else {
+            const float2 f = __half22float2(x);
+            code[e][i] = (uint32_t)uniform_code(f.x, klo[2 * i], ksc[2 * i], L) |
+                         ((uint32_t)uniform_code(f.y, klo[2 * i + 1], ksc[2 * i + 1], L) << 16);
+          }
+        }
+      }
+      if (NUQ && !sorted) {
+#pragma unroll 1
+        for (int e = 0; e < 2; ++e) {
+#pragma unroll
+          for (int i = 0; i < NH; ++i) {
+            uint32_t c = 0;
+#pragma unroll
+            for (int q = 0; q < L; ++q) {
+              const uint32_t x = e ? kx[1][i] : kx[0][i];
+              c += __hgt2_mask(*reinterpret_cast<const __half2*>(&x), *reinterpret_cast<const __half2*>(&kmu[i][q])) &
+                   0x00010001u;
+            }
+            (e ? code[1][i] : code[0][i]) = c;
+          }
+        }
+      }
+      store_codes<D, BITS>(kc, pack(code[0]), lane, true);
+      store_codes<D, BITS>(kc + ROW, pack(code[1]), lane, two);
+      kc += 2 * ROW;
+      // ---- value ranges
+      float x[2][NC], lo[2], hi[2], scale[2], u[2][NC];
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        lo[e] = INFINITY;
+        hi[e] = -INFINITY;
+#pragma unroll
+        for (int j = 0; j < NC; ++j) {
+          x[e][j] = h2f((uint16_t)(vx[e][j >> 1] >> (16 * (j & 1))));
+          lo[e] = fminf(lo[e], key[e][j] == 0u ? INFINITY : x[e][j]);
+          hi[e] = fmaxf(hi[e], key[e][j] == 0u ? -INFINITY : x[e][j]);
+        }
+        lo[e] = f32_from_key(__reduce_min_sync(0xffffffffu, f32_key(lo[e])));
+        hi[e] = f32_from_key(__reduce_max_sync(0xffffffffu, f32_key(hi[e])));
+        if (lo[e] > hi[e]) lo[e] = hi[e] = 0.f;   // no inlier
+        const float width = __fsub_rn(hi[e], lo[e]);
+        scale[e] = NUQ ? width : __fdiv_rn(width, (float)L);
+        const float rcp = __frcp_rn(scale[e]);
+#pragma unroll
+        for (int j = 0; j < NC; ++j) {
+          x[e][j] = __fsub_rn(x[e][j], lo[e]);
+          u[e][j] = div_rn(x[e][j], scale[e], rcp);
+        }
+      }
+      if (!(scale[0] > 0.f && scale[0] < INFINITY && scale[1] > 0.f && scale[1] < INFINITY)) {
+#pragma unroll
+        for (int e = 0; e < 2; ++e)
+#pragma unroll
+          for (int j = 0; j < NC; ++j) u[e][j] = scale[e] == 0.f ? 0.f : __fdiv_rn(x[e][j], scale[e]);
+      }
+      // ---- value codes
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+#pragma unroll
+        for (int i = 0; i < NH; ++i) code[e][i] = 0;
+#pragma unroll
+        for (int j = 0; j < NC; ++j) {
+          int cj;
+          if constexpr (NUQ)
+            cj = sorted ? tree_code<BITS, NC * 32>(u[e][j], top[j], s_leaf + j * 32 + lane)
+                        : count_code<BITS, NC * 32>(u[e][j], top[j], s_leaf + j * 32 + lane);
+          else
+            cj = (int)fminf(fmaxf(rintf(u[e][j]), 0.f), (float)L);
+          code[e][j >> 1] |= (uint32_t)cj << (16 * (j & 1));
+        }
+      }
+      store_codes<D, BITS>(vc, pack(code[0]), lane, true);
+      store_codes<D, BITS>(vc + ROW, pack(code[1]), lane, two);
+      vc += 2 * ROW;
+
+      // ---- key-outlier entries in channel order: (D = 128) the lanes' first pairs of channels, then
+      // their second; then the token's range and end of entries, kept by one lane and stored 32 tokens
+      // at a time
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        if (e == 1 && !two) break;
+        if (__any_sync(0xffffffffu, (om[e][0] | om[e][NH - 1]) != 0u)) {
+          const uint32_t tag = (uint32_t)((t0 + t + e) & 63) << 24;
+          auto put = [&](int32_t at, int j, uint32_t bits) {
+            if (at < cap)
+              k_out[at] = tag | ((uint32_t)chan(j) << 16) | bits;
+            else
+              atomicOr(&g_status_kvquant, MKV_FLAG_K_OUTLIER_OVERFLOW);
+          };
+#pragma unroll
+          for (int i = 0; i < NH; ++i) {
+            const bool o0 = om[e][i] & 0xffffu, o1 = om[e][i] >> 16;
+            const unsigned b0 = __ballot_sync(0xffffffffu, o0), b1 = __ballot_sync(0xffffffffu, o1);
+            if constexpr (NH == 2) {
+              const int32_t at = off + __popc(b0 & lt) + __popc(b1 & lt);
+              if (o0) put(at, 2 * i, kx[e][i] & 0xffffu);
+              if (o1) put(at + (o0 ? 1 : 0), 2 * i + 1, kx[e][i] >> 16);
+            } else {
+              if (o0) put(off + __popc(b0 & lt), 0, kx[e][i] & 0xffffu);
+              if (o1) put(off + __popc(b0) + __popc(b1 & lt), 1, kx[e][i] >> 16);
+            }
+            off += __popc(b0) + __popc(b1);
+          }
+        }
+        const int at = (t + e) & 31;
+        if (lane == at) {
+          my_off = off;
+          my_par = make_float2(lo[e], scale[e]);
+        }
+        if (at == 31 || t + e + 1 == m) {
+          if (lane <= at) {
+            off_row[t + e - at + lane] = my_off;
+            v_par[t + e - at + lane] = my_par;
+          }
+        }
+      }
+    }
+  }
+  if (t_base == 0 && blockIdx.x == 0 && threadIdx.x == 0) a.k_out_off[bh * (a.T_cap + 1)] = 0;
+  __syncthreads();                         // every thread of this CTA has read T_len
+  if (threadIdx.x == 0) {
+    const unsigned old = atomicAdd(reinterpret_cast<unsigned*>(a.T_len) + b, 1u << 24);
+    if ((int)(old >> 24) == (int)gridDim.x * a.Hkv - 1) a.T_len[b] = (int32_t)(t_base + n);
+  }
+}
+
+template <int D, int BITS>
+cudaError_t launch_bulk_t(const QuantArgs& a, int B, cudaStream_t st) {
+  // CTAs per unit: fewest (waves of two CTAs per SM) x (tokens per warp + a run's fixed cost, about
+  // eight tokens)
+  BulkSplit sp{};
+  int64_t best = INT64_MAX;
+  for (int64_t p = 1; p <= std::min<int64_t>(256 / a.Hkv, ceil_div(a.n_tokens, kBulkWarps)); ++p) {
+    const int64_t per = ceil_div(a.n_tokens, p * kBulkWarps);
+    const int64_t cost = ceil_div(p * B * a.Hkv, 2 * kNumSMs) * (per + 8);
+    if (cost < best) {
+      best = cost;
+      sp.per_w = per;
+    }
+  }
+  sp.P = (int)ceil_div(a.n_tokens, sp.per_w * kBulkWarps);
+  const dim3 grid(sp.P, B * a.Hkv);
+  quantize_count_kernel<D><<<grid, kBulkWarps * 32, 0, st>>>(a, sp);
+  const cudaError_t e = cudaPeekAtLastError();
+  if (e != cudaSuccess) return e;
+  if (a.nuq)
+    quantize_bulk_kernel<D, BITS, true><<<grid, kBulkWarps * 32, 0, st>>>(a, sp);
+  else
+    quantize_bulk_kernel<D, BITS, false><<<grid, kBulkWarps * 32, 0, st>>>(a, sp);
+  return cudaPeekAtLastError();
+}
+
+template <int D>
+cudaError_t launch_bulk_d(const QuantArgs& a, int B, cudaStream_t st) {
+  if (a.bits == 4) return launch_bulk_t<D, 4>(a, B, st);
+  if (a.bits == 3) return launch_bulk_t<D, 3>(a, B, st);
+  return launch_bulk_t<D, 2>(a, B, st);
 }
 
 // ----------------------------------------------------------------- calibrate
@@ -388,6 +916,13 @@ cudaError_t launch_quantize(const mkv_config& c, const mkv_quant_params& qp, con
   a.k_out = cache.k_out;
   a.k_out_cap = cache.k_out_cap;
   a.T_cap = cache.T_cap;
+  // Runs of tokens on many warps from kBulkMinTokens tokens on (two launches: 11 us at 64 units, 8 us at
+  // 2 units for 8 tokens); fewer (the decode step's one) take one CTA per unit, token after token (one
+  // launch: 5.0 us for one token, 10.0 / 8.5 us for 4, 13.5 / 12.0 us for 6).  The runs read fp16 rows in up to 8-byte pieces and store
+  // codes in 2-byte ones.
+  if (n_tokens >= kBulkMinTokens && ((uintptr_t)k_pre | (uintptr_t)v) % 8 == 0 &&
+      ((uintptr_t)a.k_codes | (uintptr_t)a.v_codes) % 2 == 0)
+    return c.D == 128 ? launch_bulk_d<128>(a, c.B, st) : launch_bulk_d<64>(a, c.B, st);
   const int nwords = (c.D * c.bits / 8 + 3) / 4;
   const size_t smem = 2 * c.D + 4 * c.D + 2 * nwords * 4 + 16;
   quantize_kernel<<<c.B * c.Hkv, c.D, smem, st>>>(a);
