@@ -674,71 +674,121 @@ cudaError_t launch_bulk_d(const QuantArgs& a, int B, cudaStream_t st) {
 
 // ----------------------------------------------------------------- calibrate
 
-// Per (kv-head, calibration token): value-outlier flags and u = (x - lo)/s.
-__global__ void calib_values_kernel(const __half* v_cal, int64_t N, int64_t row_stride, int D, int n_v,
-                                    float* u_out, uint8_t* vmask) {
-  extern __shared__ float absx[];
-  const int64_t ht = blockIdx.x;   // h * N + t
-  const int64_t h = ht / N, t = ht % N;
-  const int c = threadIdx.x, lane = c & 31, warp = c >> 5, nwarp = D >> 5;
-  __shared__ float s_lo[32], s_hi[32];
-  const __half xv = v_cal[(h * row_stride + t) * D + c];
-  const float x = __half2float(xv);
-  absx[c] = fabsf(x);
-  __syncthreads();
-  const float ax = absx[c];
-  int rank = 0;
-  for (int j = 0; j < D; ++j) {
-    const float o = absx[j];
-    rank += (o > ax || (o == ax && j < c)) ? 1 : 0;
+// Per (kv-head, calibration token): u = fl32((x - lo) / s) of the token's inlier values, kMasked for
+// its outliers.  One warp per token (the warp reductions of quantize_bulk_kernel).
+constexpr uint32_t kMasked = 0xffffffffu;   // no result of fp32 arithmetic has these bits
+template <int D>
+__global__ void __launch_bounds__(256) calib_values_kernel(const __half* v_cal, int64_t N, int64_t row_stride,
+                                                           int64_t n_rows, int n_v, float* u_out) {
+  constexpr int NC = D / 32;               // channels 2 NC' lane ..: pairs (2 lane, 2 lane + 1), + 64
+  const int lane = threadIdx.x & 31;
+  const int64_t ht = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (ht >= n_rows) return;
+  const __half* row = v_cal + (ht / N * row_stride + ht % N) * D;
+  uint32_t key[NC];
+  float x[NC];
+  auto chan = [&](int j) { return 2 * lane + (j & 1) + (j >> 1) * 64; };
+#pragma unroll
+  for (int j = 0; j < NC; ++j) {
+    const uint32_t b = __half_as_ushort(row[chan(j)]);
+    x[j] = h2f((uint16_t)b);
+    key[j] = ((b & 0x7fffu) << 8) | (uint32_t)(255 - chan(j));
   }
-  const bool out = rank < n_v;
-  float lo = out ? INFINITY : x, hi = out ? -INFINITY : x;
-  for (int s = 16; s > 0; s >>= 1) {
-    lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, s));
-    hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, s));
+  for (int r = 0; r < n_v; ++r) {          // the n_v largest |x| (ties: lower channel)
+    uint32_t m = key[0];
+#pragma unroll
+    for (int j = 1; j < NC; ++j) m = max(m, key[j]);
+    m = __reduce_max_sync(0xffffffffu, m);
+#pragma unroll
+    for (int j = 0; j < NC; ++j) key[j] = key[j] == m ? 0u : key[j];
   }
-  if (lane == 0) {
-    s_lo[warp] = lo;
-    s_hi[warp] = hi;
+  float lo = INFINITY, hi = -INFINITY;
+#pragma unroll
+  for (int j = 0; j < NC; ++j) {
+    lo = fminf(lo, key[j] == 0u ? INFINITY : x[j]);
+    hi = fmaxf(hi, key[j] == 0u ? -INFINITY : x[j]);
   }
-  __syncthreads();
-  lo = s_lo[0];
-  hi = s_hi[0];
-  for (int w = 1; w < nwarp; ++w) {
-    lo = fminf(lo, s_lo[w]);
-    hi = fmaxf(hi, s_hi[w]);
-  }
+  lo = f32_from_key(__reduce_min_sync(0xffffffffu, f32_key(lo)));
+  hi = f32_from_key(__reduce_max_sync(0xffffffffu, f32_key(hi)));
   if (lo > hi) lo = hi = 0.f;
   const float s = __fsub_rn(hi, lo);
-  const float u = s == 0.f ? 0.f : __fdiv_rn(__fsub_rn(x, lo), s);
-  u_out[(h * N + t) * D + c] = u;
-  vmask[(h * N + t) * D + c] = out ? 1 : 0;
+#pragma unroll
+  for (int j = 0; j < NC; ++j) {
+    const float u = s == 0.f ? 0.f : __fdiv_rn(__fsub_rn(x[j], lo), s);
+    u_out[ht * D + chan(j)] = key[j] == 0u ? __uint_as_float(kMasked) : u;
+  }
 }
 
-// Bitonic sort of n <= 4096 floats in shared memory (padded with +inf to a power of two).
-__device__ void block_sort(float* s, int n_pow2) {
-  for (int k = 2; k <= n_pow2; k <<= 1) {
-    for (int j = k >> 1; j > 0; j >>= 1) {
-      for (int i = threadIdx.x; i < n_pow2; i += blockDim.x) {
-        const int ixj = i ^ j;
-        if (ixj > i) {
-          const float a = s[i], b = s[ixj];
-          const bool up = (i & k) == 0;
-          if ((a > b) == up) {
-            s[i] = b;
-            s[ixj] = a;
-          }
-        }
-      }
+// Ascending sort of the CTA's kCalThr * E values, value i = thread * E + e (blocked): a bitonic network
+// whose merges begin with the mirrored comparison (i against i ^ (k - 1)), so every comparison puts the
+// smaller value at the lower index.  Partners in the same thread meet in registers, in the same warp
+// through shuffles, else through shared memory (sx, kCalThr * E floats).
+constexpr int kCalThr = 512;
+template <int E>
+__device__ __forceinline__ void calib_sort(float (&v)[E], float* sx) {
+  const int t = threadIdx.x;
+  // the values of thread t ^ tm, element e from e (or mirrored): the smaller or the larger one stays
+  auto exchange = [&](int tm, bool mirror, bool lower) {
+    float o[E];
+    if (tm < 32) {
+#pragma unroll
+      for (int e = 0; e < E; ++e) o[e] = __shfl_xor_sync(0xffffffffu, mirror ? v[E - 1 - e] : v[e], tm);
+    } else {
       __syncthreads();
+#pragma unroll
+      for (int e = 0; e < E; ++e) sx[e * kCalThr + t] = v[e];
+      __syncthreads();
+#pragma unroll
+      for (int e = 0; e < E; ++e) o[e] = sx[(mirror ? E - 1 - e : e) * kCalThr + (t ^ tm)];
     }
+#pragma unroll
+    for (int e = 0; e < E; ++e) v[e] = (v[e] < o[e]) == lower ? v[e] : o[e];
+  };
+  auto in_thread = [&](int m) {            // compare e with e ^ m
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      if ((e ^ m) > e) {
+        const float x = v[e], y = v[e ^ m];
+        v[e] = fminf(x, y);
+        v[e ^ m] = fmaxf(x, y);
+      }
+    }
+  };
+#pragma unroll
+  for (int k = 2; k <= E; k <<= 1) {
+    in_thread(k - 1);
+#pragma unroll
+    for (int j = k / 4; j > 0; j >>= 1) in_thread(j);
+  }
+#pragma unroll 1
+  for (int kt = 2; kt <= kCalThr; kt <<= 1) {   // merges of runs of kt threads' values
+    exchange(kt - 1, true, (t & (kt / 2)) == 0);
+#pragma unroll 1
+    for (int j = kt / 4; j > 0; j >>= 1) exchange(j, false, (t & j) == 0);
+#pragma unroll
+    for (int j = E / 2; j > 0; j >>= 1) in_thread(j);
   }
 }
 
 __device__ uint16_t fp16_next_up(uint16_t bits) {
   if (bits == 0x8000u || bits == 0u) return 0x0001u;
   return (bits & 0x8000u) ? (uint16_t)(bits - 1u) : (uint16_t)(bits + 1u);
+}
+
+// Centroids rounded to fp16: sorted by value, then made strictly increasing.
+__device__ void finish_codebook(int K, uint16_t* cb) {
+  for (int j = 1; j < K; ++j) {
+    const uint16_t v = cb[j];
+    int m = j - 1;
+    while (m >= 0 && __hgt(__ushort_as_half(cb[m]), __ushort_as_half(v))) {
+      cb[m + 1] = cb[m];
+      --m;
+    }
+    cb[m + 1] = v;
+  }
+  for (int j = 1; j < K; ++j) {
+    if (__hle(__ushort_as_half(cb[j]), __ushort_as_half(cb[j - 1]))) cb[j] = fp16_next_up(cb[j - 1]);
+  }
 }
 
 // 1-D Lloyd k-means on sorted data x[0..n): quantile start, 25 iterations,
@@ -780,30 +830,103 @@ __device__ void lloyd_codebook(const float* x, int n, int K, uint16_t* out, doub
     __syncthreads();
   }
   if (tid == 0) {
-    uint16_t cb[16];
-    for (int j = 0; j < K; ++j) cb[j] = __half_as_ushort(__double2half(cent[j]));
-    // insertion sort by value (fp16 compare)
-    for (int j = 1; j < K; ++j) {
-      const uint16_t v = cb[j];
-      int m = j - 1;
-      while (m >= 0 && __hgt(__ushort_as_half(cb[m]), __ushort_as_half(v))) {
-        cb[m + 1] = cb[m];
-        --m;
-      }
-      cb[m + 1] = v;
-    }
-    for (int j = 1; j < K; ++j) {
-      if (__hle(__ushort_as_half(cb[j]), __ushort_as_half(cb[j - 1]))) cb[j] = fp16_next_up(cb[j - 1]);
-    }
-    for (int j = 0; j < K; ++j) out[j] = cb[j];
+    for (int j = 0; j < K; ++j) out[j] = __half_as_ushort(__double2half(cent[j]));
+    finish_codebook(K, out);
   }
   __syncthreads();
 }
 
+// The same codebook by one warp from the sorted data and its exact integer prefix sums
+// P[i] = sum_{e < i} x[e] * scale (mod 2^64, scale a power of two): a cluster is a run of the sorted data,
+// found by a binary search and summed by one subtraction.  Where every partial sum of lloyd_codebook is
+// exact (the caller checks), sums and therefore centroids are the same bits; they are kept in units of
+// 1 / scale.  The nearest centroid by fp64 distances is kept exactly: between centroids a < b, "b is
+// nearer" changes once along the data, and it is evaluated in fp64 on the two values around the
+// boundary found unless they are clear of the midpoint by 2^-20 of the data's magnitude; centroids
+// closer together than that, or out of order, could tie by rounding elsewhere.  In either case the warp
+// gives up (false) and the caller takes lloyd_codebook.  (fp64 runs at two lanes a clock on this chip:
+// one division and three conversions per iteration are left of it.)
+__device__ __forceinline__ bool lloyd_sorted(const float* x, const unsigned long long* P, int n, int K, float scale,
+                                             uint16_t* out) {
+  const int lane = threadIdx.x;            // centroid
+  const bool act = lane < K;
+  const float inv = 1.f / scale;
+  const float tol = fmaxf(fabsf(x[0]), fabsf(x[n - 1])) * 0x1p-20f;
+  const double tol_s = (double)tol * scale;
+  double c = 0.0;
+  float cf = 0.f;                          // the centroid itself, to fp32
+  if (act) {
+    cf = x[min(n - 1, (int)floor((lane + 0.5) * (double)n / K))];
+    c = (double)cf * scale;
+  }
+  int bnd = lane == 0 ? 0 : n;             // first value of the lane's cluster
+  for (int it = 0; it < 25; ++it) {
+    const double cp = __shfl_up_sync(0xffffffffu, c, 1);
+    const float cpf = __shfl_up_sync(0xffffffffu, cf, 1);
+    bool ok = true;
+    if (act && lane > 0) {
+      const float m = 0.5f * (cpf + cf);
+      auto search = [&](float t) {         // first i with x[i] >= t, near the last boundary if it is there
+        int lo = max(0, bnd - 32), hi = min(n, bnd + 32);
+        if (!((lo == 0 || x[lo - 1] < t) && (hi == n || x[hi] >= t))) {
+          lo = 0;
+          hi = n;
+        }
+        while (lo < hi) {
+          const int mid = (lo + hi) >> 1;
+          if (x[mid] >= t)
+            hi = mid;
+          else
+            lo = mid + 1;
+        }
+        return lo;
+      };
+      auto nearer = [&](int i) {           // (tie: the lower centroid)
+        const double xv = (double)x[i] * scale;
+        return fabs(xv - c) < fabs(xv - cp);
+      };
+      bnd = search(m);
+      const bool below = bnd == 0 || x[bnd - 1] < m - tol, above = bnd == n || x[bnd] > m + tol;
+      ok = cf - cpf > 4.f * tol;
+      if (!(below && above)) {
+        ok = ok && c - cp > 2.0 * tol_s;
+        // the midpoint to fp32 may fall on the wrong side of a value (and of its duplicates)
+        if (bnd > 0 && nearer(bnd - 1))
+          bnd = search(x[bnd - 1]);
+        else if (bnd < n && !nearer(bnd))
+          bnd = search(nextafterf(x[bnd], INFINITY));
+        ok = ok && (bnd == 0 || !nearer(bnd - 1)) && (bnd == n || nearer(bnd));
+      }
+    }
+    if (!__all_sync(0xffffffffu, ok)) return false;
+    int end = __shfl_down_sync(0xffffffffu, bnd, 1);
+    if (lane == K - 1) end = n;
+    bool same = true;
+    if (act && end > bnd) {
+      const double cn = (double)(long long)(P[end] - P[bnd]) / (double)(end - bnd);
+      same = __double_as_longlong(cn) == __double_as_longlong(c);
+      c = cn;
+      cf = (float)cn * inv;
+    }
+    if (__all_sync(0xffffffffu, same)) break;   // a fixed point: the iterations left change nothing
+  }
+  const __half h = __double2half(c * (double)inv);
+  const __half hp = __ushort_as_half((unsigned short)__shfl_up_sync(0xffffffffu, (unsigned)__half_as_ushort(h), 1));
+  if (!__all_sync(0xffffffffu, !act || lane == 0 || __hlt(hp, h))) {   // sort and nudge: one thread
+    for (int j = 0; j < K; ++j) {
+      const unsigned hj = __shfl_sync(0xffffffffu, (unsigned)__half_as_ushort(h), j);
+      if (lane == 0) out[j] = (uint16_t)hj;
+    }
+    if (lane == 0) finish_codebook(K, out);
+  } else if (act) {
+    out[lane] = __half_as_ushort(h);
+  }
+  return true;
+}
+
 struct CalibArgs {
   const __half* k_cal;   // [Hkv][row_stride][D]
-  const float* u;        // [Hkv][N][D]
-  const uint8_t* vmask;  // [Hkv][N][D]
+  const float* u;        // [Hkv][N][D], kMasked for outliers
   int64_t N, row_stride;
   int D, bits, nuq, nt, all_out;
   float* t_lo;
@@ -814,71 +937,137 @@ struct CalibArgs {
   uint16_t* v_cb;
 };
 
-// grid (Hkv*D, 2): y = 0 keys, y = 1 values (NUQ only).
-__global__ void calib_channel_kernel(const CalibArgs a) {
-  extern __shared__ float s[];   // [n_pow2] data, then fp64 centroids and assignments
+// First index of s[0..n) (ascending) whose value is >= t (or > t).
+__device__ __forceinline__ int first_at(const float* s, int n, float t, bool above) {
+  int lo = 0, hi = n;
+  while (lo < hi) {
+    const int mid = (lo + hi) >> 1;
+    if (above ? s[mid] > t : s[mid] >= t)
+      hi = mid;
+    else
+      lo = mid + 1;
+  }
+  return lo;
+}
+
+// grid (Hkv*D, 2): y = 0 keys, y = 1 values (NUQ only).  One channel per CTA: its N values sorted
+// (E per thread), prefix sums, then one warp runs Lloyd's iterations.  4 bits, N = 4096, 8 x 128
+// channels: the values' kernel 13 us, this one 240 us, the whole call 0.26 ms (55 ms with a brute-force
+// fp64 search and sequential sums on every iteration); bound by the sort's instructions (45 thousand per
+// channel) and the latency of the one warp that iterates.
+template <int E>
+__global__ void __launch_bounds__(kCalThr) calib_channel_kernel(const CalibArgs a) {
+  constexpr int NP2 = kCalThr * E;
+  extern __shared__ __align__(16) uint8_t smem[];
+  unsigned long long* P = reinterpret_cast<unsigned long long*>(smem);   // [NP2 + 2] prefix sums
+  float* s = reinterpret_cast<float*>(P + NP2 + 2);                      // [NP2]
+  __shared__ unsigned long long s_warp[kCalThr / 32];
+  __shared__ int s_cnt, s_fast, s_a, s_b;
+  __shared__ double cent[16];
   const int hc = blockIdx.x;
   const int h = hc / a.D, c = hc % a.D;
   const bool values = blockIdx.y == 1;
-  if (values && !a.nuq) return;
-  int n_pow2 = 1;
-  while (n_pow2 < a.N) n_pow2 <<= 1;
-  double* cent = reinterpret_cast<double*>(s + n_pow2 + (n_pow2 & 1));
-  uint8_t* asg = reinterpret_cast<uint8_t*>(cent + 16);
-  __shared__ int s_cnt;
-  if (threadIdx.x == 0) s_cnt = 0;
-  __syncthreads();
-  for (int i = threadIdx.x; i < n_pow2; i += blockDim.x) {
-    float v = INFINITY;
-    if (i < a.N) {
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const int N = (int)a.N, K = 1 << a.bits, L = K - 1;
+  if (t == 0) s_cnt = 0;
+  float v[E];
+  int cnt = 0;
+#pragma unroll
+  for (int e = 0; e < E; ++e) {            // any order: the values are sorted next
+    const int i = e * kCalThr + t;
+    v[e] = INFINITY;
+    if (i < N) {
       if (!values) {
-        v = __half2float(a.k_cal[((int64_t)h * a.row_stride + i) * a.D + c]);
-      } else if (!a.vmask[((int64_t)h * a.N + i) * a.D + c]) {
-        v = a.u[((int64_t)h * a.N + i) * a.D + c];
-        atomicAdd(&s_cnt, 1);
+        v[e] = __half2float(a.k_cal[((int64_t)h * a.row_stride + i) * a.D + c]);
+      } else {
+        const float u = a.u[((int64_t)h * N + i) * a.D + c];
+        if (__float_as_uint(u) != kMasked) {
+          v[e] = u;
+          ++cnt;
+        }
       }
     }
-    s[i] = v;
+  }
+  calib_sort<E>(v, s);
+  __syncthreads();
+#pragma unroll
+  for (int e = 0; e < E; ++e) s[t * E + e] = v[e];
+  if (values) {
+    cnt = __reduce_add_sync(0xffffffffu, cnt);
+    if (lane == 0) atomicAdd(&s_cnt, cnt);
+  }
+  // exact prefix sums: keys are multiples of 2^-24; normalized values of at least 2^-18 (checked
+  // below) multiples of 2^-41
+  const float scale = values ? 0x1p41f : 0x1p24f;
+  unsigned long long q[E], run = 0;
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    q[e] = run;
+    run += (unsigned long long)__float2ll_rn(v[e] * scale);
+  }
+  unsigned long long incl = run;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned long long y = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += y;
+  }
+  if (lane == 31) s_warp[warp] = incl;
+  __syncthreads();
+  unsigned long long base = incl - run;
+  for (int w = 0; w < warp; ++w) base += s_warp[w];
+#pragma unroll
+  for (int e = 0; e < E; ++e) P[t * E + e] = base + q[e];
+  if (t == kCalThr - 1) P[NP2] = base + run;
+  __syncthreads();
+  if (warp == 0) {
+    int ia = 0, ib = s_cnt;
+    if (!values) {
+      float tl = INFINITY, th = -INFINITY;
+      ib = 0;
+      if (!a.all_out) {                    // inliers: the sorted range with tl <= x <= th
+        tl = s[a.nt];
+        th = s[N - 1 - a.nt];
+        ia = first_at(s, N, tl, false);
+        ib = first_at(s, N, th, true);
+      }
+      if (lane == 0) {
+        a.t_lo[hc] = tl;
+        a.t_hi[hc] = th;
+        const float lo = a.all_out ? 0.f : tl, hi = a.all_out ? 0.f : th;
+        if (a.k_lo) a.k_lo[hc] = lo;
+        if (a.k_scale) a.k_scale[hc] = __fdiv_rn(__fsub_rn(hi, lo), (float)L);
+      }
+    }
+    bool fast = a.nuq && ib > ia;
+    if (fast) {                            // finite; keys: |sums| < 2^28; values: in [0, 1], none in (0, 2^-18)
+      fast = s[ia] > -INFINITY && s[ib - 1] < INFINITY;
+      if (values) {
+        const int z = first_at(s, ib, 0.f, true);
+        fast = fast && s[ia] >= 0.f && s[ib - 1] <= 1.f && (z == ib || s[z] >= 0x1p-18f);
+      }
+    }
+    if (fast)
+      fast = lloyd_sorted(s + ia, P + ia, ib - ia, K, scale,
+                          (values ? a.v_cb : a.k_cb) + (int64_t)hc * K);
+    if (lane == 0) {
+      s_fast = fast;
+      s_a = ia;
+      s_b = ib;
+    }
   }
   __syncthreads();
-  block_sort(s, n_pow2);
-  const int K = 1 << a.bits, L = K - 1;
-  if (!values) {
-    const int N = (int)a.N;
-    float tl = INFINITY, th = -INFINITY;
-    if (!a.all_out) {
-      tl = s[a.nt];
-      th = s[N - 1 - a.nt];
-    }
-    if (threadIdx.x == 0) {
-      a.t_lo[hc] = tl;
-      a.t_hi[hc] = th;
-      const float lo = a.all_out ? 0.f : tl, hi = a.all_out ? 0.f : th;
-      if (a.k_lo) a.k_lo[hc] = lo;
-      if (a.k_scale) a.k_scale[hc] = __fdiv_rn(__fsub_rn(hi, lo), (float)L);
-    }
-    if (a.nuq) {
-      // inliers: the contiguous sorted range with tl <= x <= th
-      __shared__ int s_a, s_b;
-      if (threadIdx.x == 0) {
-        int lo_i = 0, hi_i = 0;
-        if (!a.all_out) {
-          lo_i = a.nt;
-          while (lo_i > 0 && s[lo_i - 1] >= tl) --lo_i;
-          hi_i = N - 1 - a.nt;
-          while (hi_i + 1 < N && s[hi_i + 1] <= th) ++hi_i;
-          hi_i += 1;
-        }
-        s_a = lo_i;
-        s_b = hi_i;
-      }
-      __syncthreads();
-      lloyd_codebook(s + s_a, s_b - s_a, K, a.k_cb + (int64_t)hc * K, cent, asg);
-    }
-  } else {
-    __syncthreads();
-    lloyd_codebook(s, s_cnt, K, a.v_cb + (int64_t)hc * K, cent, asg);
-  }
+  if (a.nuq && !s_fast)                    // the prefix sums' room takes the assignments
+    lloyd_codebook(s + s_a, s_b - s_a, K, (values ? a.v_cb : a.k_cb) + (int64_t)hc * K, cent,
+                   reinterpret_cast<uint8_t*>(P));
+}
+
+template <int E>
+cudaError_t launch_calib_t(const CalibArgs& a, int channels, cudaStream_t st) {
+  constexpr int smem = (kCalThr * E + 2) * 8 + kCalThr * E * 4;
+  const cudaError_t e = cudaFuncSetAttribute(calib_channel_kernel<E>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  calib_channel_kernel<E><<<dim3(channels, a.nuq ? 2 : 1), kCalThr, smem, st>>>(a);
+  return cudaPeekAtLastError();
 }
 
 }  // namespace
@@ -934,15 +1123,16 @@ cudaError_t launch_calibrate(const mkv_config& c, const void* k_cal, const void*
   const bool nuq = c.quant_mode == MKV_QUANT_NUQ;
   const int n_v = std::min(c.D, (int)ceil((double)c.outlier_frac * c.D));
   if (nuq) {
-    calib_values_kernel<<<(unsigned)(c.Hkv * N), c.D, c.D * sizeof(float), st>>>(
-        static_cast<const __half*>(v_cal), N, row_stride, c.D, n_v, ws.u, ws.vmask);
+    const int64_t rows = (int64_t)c.Hkv * N;
+    auto values = c.D == 128 ? calib_values_kernel<128> : calib_values_kernel<64>;
+    values<<<(unsigned)ceil_div(rows, 8), 256, 0, st>>>(static_cast<const __half*>(v_cal), N, row_stride, rows, n_v,
+                                                        ws.u);
     cudaError_t e = cudaPeekAtLastError();
     if (e != cudaSuccess) return e;
   }
   CalibArgs a{};
   a.k_cal = static_cast<const __half*>(k_cal);
   a.u = ws.u;
-  a.vmask = ws.vmask;
   a.N = N;
   a.row_stride = row_stride;
   a.D = c.D;
@@ -956,14 +1146,12 @@ cudaError_t launch_calibrate(const mkv_config& c, const void* k_cal, const void*
   a.k_scale = qp.k_scale;
   a.k_cb = qp.k_cb;
   a.v_cb = qp.v_cb;
-  int n_pow2 = 1;
-  while (n_pow2 < N) n_pow2 <<= 1;
-  const size_t smem = (size_t)(n_pow2 + 2) * sizeof(float) + 16 * sizeof(double) + n_pow2 + 16;
-  cudaError_t e = cudaFuncSetAttribute(calib_channel_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
-  if (e != cudaSuccess) return e;
-  calib_channel_kernel<<<dim3(c.Hkv * c.D, nuq ? 2 : 1), 512, smem, st>>>(a);
-  return cudaPeekAtLastError();
+  // values per thread: the smallest power of two that holds N
+  const int channels = c.Hkv * c.D;
+  if (N <= kCalThr) return launch_calib_t<1>(a, channels, st);
+  if (N <= 2 * kCalThr) return launch_calib_t<2>(a, channels, st);
+  if (N <= 4 * kCalThr) return launch_calib_t<4>(a, channels, st);
+  return launch_calib_t<8>(a, channels, st);
 }
 
 cudaError_t take_status_kvquant(uint32_t* flags, cudaStream_t st) {

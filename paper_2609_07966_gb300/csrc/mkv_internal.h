@@ -68,9 +68,9 @@ PrefillWs prefill_ws(const mkv_config& c, int64_t T, void* base);
 
 // Calibration workspace (KVQuant).
 struct CalibWs {
-  float* sorted;   // [Hkv][D][N] sorted calibration values (keys or u)
-  float* u;        // [Hkv][N][D] normalized values
-  uint8_t* vmask;  // [Hkv][N][D] value-outlier flags
+  float* sorted;   // [Hkv][D][N] not used (the documented workspace size stays)
+  float* u;        // [Hkv][N][D] normalized values, value outliers marked
+  uint8_t* vmask;  // [Hkv][N][D] not used
   size_t bytes;
 };
 CalibWs calib_ws(const mkv_config& c, int64_t N, void* base);
