@@ -70,7 +70,8 @@ typedef enum { MKV_QUANT_UNIFORM = 0, MKV_QUANT_NUQ = 1 } mkv_quant_mode;
 #define MKV_FLAG_K_OUTLIER_OVERFLOW 0x1u  /* a key-outlier CSR region is full */
 #define MKV_FLAG_CACHE_FULL 0x2u          /* an append found no free slot; dropped */
 #define MKV_FLAG_WAIT_TIMEOUT 0x4u        /* a prefill-scoring CTA gave up waiting on the
-                                             tensor core; that call's scores are invalid */
+                                             tensor core, or a RocketKV step's CTA on its
+                                             cluster; that call's results are invalid */
 
 /* One configuration (a row of Table 1, with its parameters).  Host POD. */
 typedef struct {
@@ -396,9 +397,9 @@ mkv_status mkv_rocket_select(const mkv_config* cfg, const void* q, const mkv_cac
 /* RocketKV decode step in one launch: the page choice of mkv_rocket_select
  * and the sparse exact attention of mkv_decode_attention over the chosen
  * pages plus the newest token's page (Section 2.1, RocketKV paragraph, stage
- * 2).  One cluster of 8 CTAs per (batch, kv-head) exchanges page scores and
+ * 2).  A cluster of 1 to 8 CTAs per (batch, kv-head) exchanges page scores and
  * attention partials through distributed shared memory, so no workspace is
- * needed.  q fp16 [B][Hq][D]; out fp16 [B][Hq][D]; page_idx_out (optional,
+ * needed (a bounded wait on them that ran out sets MKV_FLAG_WAIT_TIMEOUT).  q fp16 [B][Hq][D]; out fp16 [B][Hq][D]; page_idx_out (optional,
  * NULL to skip) int32 [B][Hkv][topk_pages] as mkv_rocket_select writes it.
  * The page scores are the same sums in another fp32 order, so a near-tie
  * may pick another page than mkv_rocket_select.  MKV_ERR_UNSUPPORTED when

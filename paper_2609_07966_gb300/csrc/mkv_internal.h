@@ -133,11 +133,12 @@ cudaError_t launch_snap_keep(const mkv_config& c, const void* full_k, const void
 cudaError_t launch_rocket_select(const mkv_config& c, const void* q, const mkv_cache& cache,
                                  int32_t* page_idx, cudaStream_t st);
 // Fused RocketKV step (page choice + sparse attention, one cluster per (batch, kv-head)).
+// The bytes that decide whether a cache length is accepted.
 size_t rocket_fused_smem(const mkv_config& c, int64_t T_cap);
 // k_new / v_new: the step's token, appended by the same launch (null: no append).
 cudaError_t launch_rocket_fused(const mkv_config& c, const void* q, const mkv_cache& cache, int32_t* page_idx,
                                 void* out, const void* k_new, const void* v_new, cudaStream_t st);
-constexpr int kRocketCluster = 8;   // CTAs of the fused step per (batch, kv-head)
+constexpr int kRocketCluster = 8;   // most CTAs of the fused step per (batch, kv-head)
 
 // Host-side argument checks of an FP16 decode call (config, cache, q/out pointers).
 mkv_status check_fp16_decode_args(const mkv_config* cfg, const mkv_cache* cache, const void* q, const void* out);

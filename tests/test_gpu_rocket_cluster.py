@@ -1,0 +1,55 @@
+"""GPU: the one-launch RocketKV step at every cluster size and where its page choice could go wrong
+(tied and equal scores, one page to several thousand, budgets from one page to all of them) against the
+two calls it stands for: mkv_rocket_select must list the same pages (integer inputs make the scores
+exact in any order) and mkv_decode_attention over them agree within the attention tolerance."""
+import numpy as np
+import pytest
+
+import paper_2609_07966_gb300 as mkv
+from paper_2609_07966_gb300 import caches
+
+from gpu_util import assert_close, to_dev, torch_cuda
+
+pytestmark = pytest.mark.gpu
+
+CASES = [  # B, Hq, Hkv, D, slots held, slots, pages chosen, dims, values
+    (1, 8, 8, 128, 4097, 4160, 64, 32, "ties"), (3, 32, 8, 128, 700, 720, 9, 32, "ties"),
+    (9, 32, 8, 128, 1040, 1056, 20, 40, "plain"), (10, 8, 8, 64, 333, 336, 5, 16, "ties"),
+    (15, 16, 8, 64, 4112, 4128, 100, 16, "ties"), (20, 32, 8, 128, 500, 512, 40, 32, "plain"),
+    (1, 8, 1, 128, 16400, 16432, 257, 128, "ties"), (1, 8, 2, 64, 40000, 40016, 300, 3, "ties"),
+    (2, 8, 2, 64, 777, 784, 48, 16, "equal"), (130, 1, 1, 64, 2000, 2000, 11, 16, "equal"),
+    (1, 2, 2, 128, 1, 16, 4, 8, "plain"), (1, 4, 2, 64, 16, 32, 4, 8, "plain"), (2, 4, 2, 64, 17, 32, 1, 8, "plain"),
+]
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,D,n,cap,pages,dims,values", CASES)
+def test_fused_equals_two_calls(B, Hq, Hkv, D, n, cap, pages, dims, values):
+    torch = torch_cuda()
+    dev = torch.device("cuda")
+    rng = np.random.default_rng(n + B)
+    if values == "plain":
+        k = rng.integers(-9, 10, (B, Hkv, cap, D)) / 8
+    else:
+        k = rng.integers(0 if values == "equal" else -1, 1 if values == "equal" else 2, (B, Hkv, cap, D)) * 1.0
+    q = rng.integers(-3, 4, (B, Hq, D)) / 4
+    cfg = mkv.config(mkv.MKV_ROCKET, B, Hq, Hkv, D, snap_window=1, snap_keep=cap, topk_pages=pages, topq_dims=dims)
+    c = caches.alloc_cache(cfg, cap, device=dev)
+    c.t["k"].copy_(to_dev(k.astype(np.float16), dev))
+    c.t["v"].normal_(generator=torch.Generator(device=dev).manual_seed(n))
+    pg = c.t["k"].unflatten(2, (cap // 16, 16))
+    c.t["kmin"].copy_(pg.amin(3).transpose(2, 3))
+    c.t["kmax"].copy_(pg.amax(3).transpose(2, 3))
+    c.t["T_len"].fill_(n)
+    if B > 2:
+        c.t["T_len"][1] = 0                                 # an empty entry and a short one
+        c.t["T_len"][2] = min(n, 20)
+    qd = to_dev(q.astype(np.float16), dev)
+    ws, nws = caches.workspace(cfg, cap, device=dev)
+    idx, idx2 = (torch.full((B, Hkv, pages), -7, dtype=torch.int32, device=dev) for _ in range(2))
+    out, out2 = torch.empty_like(qd), torch.empty_like(qd)
+    mkv.mkv_rocket_select(cfg, qd.data_ptr(), c.c, idx.data_ptr())
+    mkv.mkv_decode_attention(cfg, qd.data_ptr(), c.c, None, idx.data_ptr(), out.data_ptr(), ws.data_ptr(), nws)
+    mkv.mkv_rocket_decode(cfg, qd.data_ptr(), c.c, idx2.data_ptr(), out2.data_ptr())
+    assert torch.equal(idx, idx2)
+    assert_close(out2.float().cpu(), out.float().cpu(), "fused against two calls")
+    assert mkv.mkv_get_status() == 0
