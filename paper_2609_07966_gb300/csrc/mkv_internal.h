@@ -125,6 +125,7 @@ cudaError_t launch_h2o_update(const mkv_config& c, const mkv_cache& cache, const
                               cudaStream_t st);
 cudaError_t launch_prefill_scores(const mkv_config& c, const void* q, int64_t q_rows, int64_t T,
                                   const void* full_k, const PrefillWs& ws, cudaStream_t st);
+float* prefill_second_sums(const mkv_config& c, int64_t q_rows, const PrefillWs& ws);
 cudaError_t launch_h2o_keep(const mkv_config& c, const void* full_k, const void* full_v, int64_t T,
                             const mkv_cache& cache, const PrefillWs& ws, cudaStream_t st);
 cudaError_t launch_snap_keep(const mkv_config& c, const void* full_k, const void* full_v, int64_t T,

@@ -87,6 +87,7 @@ struct ScoreArgs {
   float scale_log2;
   float2* row_st;       // [B Hkv][rowblocks][n_ksplit][128]: pass 1's (m, l); merged at split 0 (rowmerge_kernel)
   float* score;         // [B Hkv][T]
+  float* score2;        // one query block: the sums of its second 64 rows (or null: added onto a zeroed score)
 };
 
 template <int D, int TN>
@@ -485,9 +486,12 @@ __global__ void __launch_bounds__(kThr, 1)
 // ---------------------------------------------------------------- pass 2 over one query block
 // When the query rows fit one 128-row block (an observation window of at most 128 / G rows), pass 2's
 // CTAs would each meet a single tile; instead a CTA holds the query block and its statistics (the
-// MMA's B) and streams a run of 128-key tiles as the MMA's A.  Each key's sum over the block's rows
-// comes from the two column halves of the tile and is added to the zeroed score (two float adds onto
-// 0, so the result does not depend on their order).
+// MMA's B) and streams a run of 128-key tiles as the MMA's A.  The runs are pass 1's key splits, taken
+// from their ends: what pass 1 read last is still in L2 (SnapKV 32K, batch 4: 268 MB of keys, 129 MB of
+// L2; 186 MB are read from HBM).  One wave of 4 x 32 CTAs streams them in 44 us where 5 x 32 on 152 SMs
+// took two waves (pass 1: 44-55 us; both were about 74 us).  Each CTA merges its unit's row statistics itself.  A key's sum over the block's rows comes from
+// the two column halves of the tile: into score and score2, or added to the zeroed score (two float adds
+// onto 0; the same sum in either order).
 template <int D>
 __global__ void __launch_bounds__(kThr, 1)
     colsum_window_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant__ CUtensorMap kmap,
@@ -505,25 +509,40 @@ __global__ void __launch_bounds__(kThr, 1)
   const int lr = lq * 32 + (threadIdx.x & 31);           // accumulator lane = key of the tile
   const int64_t t_begin = (int64_t)blockIdx.x * tiles_per_cta;
   const int ntiles = (int)std::max<int64_t>(0, std::min<int64_t>(ceil_div_dev(a.T, kBlk) - t_begin, tiles_per_cta));
-  const float2* stats = a.row_st + (int64_t)bh * a.n_ksplit * kTM;   // the unit's one block, split 0
+  const int64_t t_last = t_begin + ntiles - 1;
+  // the block's row statistics, merged over pass 1's key splits as rowmerge_kernel does
+  if (threadIdx.x < kBlk) {
+    const int c = threadIdx.x;
+    const float2* p = a.row_st + (int64_t)bh * a.n_ksplit * kTM + c;
+    float M = -INFINITY;
+    for (int s = 0; s < a.n_ksplit; ++s) M = fmaxf(M, p[s * kBlk].x);
+    float Ls = 0.f;
+    for (int s = 0; s < a.n_ksplit; ++s) {
+      const float2 x = p[s * kBlk];
+      if (x.x != -INFINITY) Ls += x.y * exp2f(x.x - M);
+    }
+    const bool valid = (c & (a.rpb - 1)) < a.R && M != -INFINITY && Ls > 0.f;
+    float* out = reinterpret_cast<float*>(sm + L::ST_OFF);
+    out[(c >> 1) * 4 + (c & 1)] = valid ? -M : -INFINITY;
+    out[(c >> 1) * 4 + 2 + (c & 1)] = valid ? 1.f / Ls : 0.f;
+  }
 
   const uint32_t tbase = cta_setup(ctl);
   run_roles<D, kTN2, false, true>(
       sm, ctl, tbase, ntiles,
-      [&](uint64_t* bar) {                // the query block and its statistics
-        tc_mbar_expect_tx(bar, L::TILE_A + kStatBytes);
+      [&](uint64_t* bar) {                // the query block
+        tc_mbar_expect_tx(bar, L::TILE_A);
         for (int at = 0; at < D / 64; ++at)
           tma_load_4d(sm + L::A_OFF + at * L::ATOM_A, &qmap, at * 64, 0, kvh * a.G, b, bar);
-        bulk_load(sm + L::ST_OFF, stats, kStatBytes, bar);
       },
       [&](int t, int s, uint64_t* bar) {  // 128 keys
         tc_mbar_expect_tx(bar, L::TILE_B);
         for (int at = 0; at < D / 64; ++at)
-          tma_load_4d(sm + L::B_OFF + s * L::TILE_B + at * L::ATOM_B, &kmap, at * 64, (int)((t_begin + t) * kBlk),
+          tma_load_4d(sm + L::B_OFF + s * L::TILE_B + at * L::ATOM_B, &kmap, at * 64, (int)((t_last - t) * kBlk),
                       kvh, b, bar);
       },
       [&](int t, uint32_t col, int) {
-        const int64_t jt = (t_begin + t) * kBlk;
+        const int64_t jt = (t_last - t) * kBlk;
         const int64_t jrel = jt + lr - a.pos0;   // rows i >= jrel see this key
         const float4* s4 = reinterpret_cast<const float4*>(sm + L::ST_OFF) + hf * 32;
         const uint64_t sc2 = pk2(a.scale_log2, a.scale_log2);
@@ -549,7 +568,14 @@ __global__ void __launch_bounds__(kThr, 1)
           }
         }
         const float2 s0 = upk2(sp2[0]), s1 = upk2(sp2[1]);
-        if (jt + lr < a.T) atomicAdd(a.score + (int64_t)bh * a.T + jt + lr, (s0.x + s0.y) + (s1.x + s1.y));
+        const float sum = (s0.x + s0.y) + (s1.x + s1.y);
+        if (jt + lr < a.T) {
+          const int64_t at = (int64_t)bh * a.T + jt + lr;
+          if (a.score2 != nullptr)
+            (hf ? a.score2 : a.score)[at] = sum;
+          else
+            atomicAdd(a.score + at, sum);
+        }
       });
   cta_teardown(ctl, tbase);
 }
@@ -601,19 +627,17 @@ cudaError_t launch_scores_t(const CUtensorMap& qm, const CUtensorMap& k256, cons
   rowstats_tc_kernel<D><<<dim3(a.n_ksplit, a.rowblocks, units), kThr, smem1, st>>>(qm, k256, a);
   e = cudaPeekAtLastError();
   if (e != cudaSuccess) return e;
+  if (a.rowblocks == 1) {                 // one query block: hold it, stream pass 1's key splits
+    e = cudaFuncSetAttribute(colsum_window_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem2);
+    if (e == cudaSuccess && a.score2 == nullptr) e = cudaMemsetAsync(a.score, 0, (size_t)units * a.T * sizeof(float), st);
+    if (e != cudaSuccess) return e;
+    colsum_window_kernel<D><<<dim3(a.n_ksplit, units), kThr, smem2, st>>>(qm, k128, a, a.tiles_per_split * (kTN1 / kBlk));
+    return cudaPeekAtLastError();
+  }
   rowmerge_kernel<<<(unsigned)((int64_t)units * a.rowblocks), kBlk, 0, st>>>(a.row_st, a.n_ksplit, a.rpb,
                                                                             a.rowblocks, a.R);
   e = cudaPeekAtLastError();
   if (e != cudaSuccess) return e;
-  if (a.rowblocks == 1) {                 // one query block: hold it, stream runs of key tiles
-    e = cudaFuncSetAttribute(colsum_window_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem2);
-    if (e == cudaSuccess) e = cudaMemsetAsync(a.score, 0, (size_t)units * a.T * sizeof(float), st);
-    if (e != cudaSuccess) return e;
-    const int64_t per = ceil_div((int64_t)keyblocks, ceil_div(kNumSMs, (int64_t)units));
-    colsum_window_kernel<D><<<dim3((unsigned)ceil_div((int64_t)keyblocks, per), units), kThr, smem2, st>>>(
-        qm, k128, a, (int)per);
-    return cudaPeekAtLastError();
-  }
   colsum_tc_kernel<D><<<dim3(keyblocks, units), kThr, smem2, st>>>(qm, k128, a);
   return cudaPeekAtLastError();
 }
@@ -638,6 +662,12 @@ cudaError_t launch_wait_selftest(int ms, cudaStream_t st) {
   return cudaPeekAtLastError();
 }
 
+// RocketKV, one query block: the keep list's room (written only after the scores are read) takes the sums
+// of the block's second 64 rows; snap_keep_kernel adds the two.  Null: score is complete.
+float* prefill_second_sums(const mkv_config& c, int64_t q_rows, const PrefillWs& ws) {
+  return c.method == MKV_ROCKET && q_rows <= kTM / (c.Hq / c.Hkv) ? reinterpret_cast<float*>(ws.keep) : nullptr;
+}
+
 cudaError_t launch_prefill_scores(const mkv_config& c, const void* q, int64_t q_rows, int64_t T,
                                   const void* full_k, const PrefillWs& ws, cudaStream_t st) {
   if (q_rows <= 0 || T <= 0) return cudaSuccess;
@@ -655,15 +685,28 @@ cudaError_t launch_prefill_scores(const mkv_config& c, const void* q, int64_t q_
   const int units = c.B * c.Hkv;
   const int64_t tiles = ceil_div(T, kTN1);               // pass 1's key tiles
   if (a.rowblocks > 65535 || T > INT32_MAX - kTN1) return cudaErrorInvalidConfiguration;
-  // split the key range only when the row blocks are fewer than the SMs (an observation window);
-  // the splits' partials stay within the row-statistics workspace of B Hq (T + 128) entries
-  int64_t ns = ceil_div(kNumSMs, (int64_t)a.rowblocks * units);
-  ns = std::min<int64_t>(ns, std::min<int64_t>(tiles, (T + kTM) / ((int64_t)a.rowblocks * a.rpb)));
-  ns = std::max<int64_t>(ns, 1);
+  // split the key range only when the row blocks are fewer than the SMs (an observation window): the
+  // split that takes the fewest (waves of one CTA per SM) x (tiles + a CTA's fixed cost, about four
+  // tiles); the splits' partials stay within the row-statistics workspace of B Hq (T + 128) entries
+  const int64_t blocks = (int64_t)a.rowblocks * units;
+  int64_t ns = 1;
+  if (blocks < kNumSMs) {
+    const int64_t most = std::max<int64_t>(
+        1, std::min<int64_t>({tiles, (T + kTM) / ((int64_t)a.rowblocks * a.rpb), 2 * kNumSMs}));
+    int64_t best = INT64_MAX;
+    for (int64_t n = 1; n <= most; ++n) {
+      const int64_t cost = ceil_div(blocks * n, kNumSMs) * (ceil_div(tiles, n) + 4);
+      if (cost < best) {
+        best = cost;
+        ns = n;
+      }
+    }
+  }
   a.tiles_per_split = (int)ceil_div(tiles, ns);
   a.n_ksplit = (int)ceil_div(tiles, a.tiles_per_split);
   a.row_st = ws.row_st;
   a.score = ws.score;
+  a.score2 = prefill_second_sums(c, q_rows, ws);
   CUtensorMap qm, k256, k128;
   // q [B][Hq][R][D] in boxes of G heads x rpb rows; k [B][Hkv][T][D] in 256- and 128-key boxes
   cudaError_t e = make_map(&qm, q, c.D, q_rows, c.Hq, c.B, a.rpb, a.G);
