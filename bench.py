@@ -271,7 +271,7 @@ class Runner:
                 self.rocket_fused = t_fused <= t_split
 
     def choose_kvquant_step(self, reps=3):
-        """KVQuant: the one-launch step (mkv_kvquant_step) or quantize + decode, whichever is faster on
+        """KVQuant: the one-call step (mkv_kvquant_step) or quantize + decode, whichever is faster on
         this shape (both leave the same cache and output bits); a few eager steps of each, timed with
         CUDA events.  Returns both times (ms per step)."""
         torch = self.torch
@@ -289,8 +289,8 @@ class Runner:
             torch.cuda.synchronize()
             t[fused] = e0.elapsed_time(e1) / reps
         self.step_fused = t[True] <= t[False]
-        return {"one_launch_step": t[True], "quantize_then_decode": t[False],
-                "chosen": "one_launch_step" if self.step_fused else "quantize_then_decode"}
+        return {"kvquant_step": t[True], "quantize_then_decode": t[False],
+                "chosen": "kvquant_step" if self.step_fused else "quantize_then_decode"}
 
     def append(self, l, kn=None, vn=None):
         mkv = self.mkv
@@ -409,7 +409,7 @@ class Runner:
     def launches_per_step(self):
         # per layer: FP16 / H2O / KVQuant append (KVQuant: quantize) and attention in one launch (H2O:
         # + score update); RocketKV append, page choice and attention in one launch
-        per = {"fp16": 1 if self.step_fused else 2, "kvquant": 1 if self.step_fused else 2,
+        per = {"fp16": 1 if self.step_fused else 2, "kvquant": 2,
                "h2o": 2 if self.step_fused else 3,
                "rocket": 1 if self.rocket_fused else 3}[self.method]
         return per * self.w.L

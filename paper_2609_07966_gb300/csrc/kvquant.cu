@@ -63,6 +63,8 @@ struct QuantArgs {
   uint32_t* k_out;       // [B][Hkv][k_out_cap]
   int64_t k_out_cap;
   int64_t T_cap;
+  int trigger;           // let the decode of the same step start (mkv_kvquant_step)
+  int tickets;           // 0: more kv-heads than the tickets in T_len's top 8 bits count; advance_kernel follows
 };
 
 // One CTA per (batch, kv-head), one thread per channel; tokens in order so the
@@ -70,6 +72,8 @@ struct QuantArgs {
 // last CTA of batch entry b to finish stores the new length: during the launch
 // the top 8 bits of T_len[b] count the finished CTAs (readers mask them off).
 __global__ void quantize_kernel(const QuantArgs a) {
+  asm volatile("griddepcontrol.wait;\n" ::: "memory");   // (no-op in a plain launch)
+  if (a.trigger) asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
   extern __shared__ uint8_t sm[];
   const int D = a.D, K = 1 << a.bits, L = K - 1;
   const int bh = blockIdx.x;
@@ -109,7 +113,7 @@ __global__ void quantize_kernel(const QuantArgs a) {
   // the last CTA of batch entry b stores its new length (after every thread of this CTA read it)
   auto finish = [&](int64_t len) {
     __syncthreads();
-    if (c == 0) {
+    if (c == 0 && a.tickets) {
       const unsigned old = atomicAdd(reinterpret_cast<unsigned*>(a.T_len) + b, 1u << 24);
       if ((int)(old >> 24) == a.Hkv - 1) a.T_len[b] = (int32_t)len;
     }
@@ -144,6 +148,12 @@ __global__ void quantize_kernel(const QuantArgs a) {
                          scr, &g_status_kvquant, [] { __syncthreads(); });
   }
   finish(t_base + a.n_tokens);
+}
+
+// The new lengths where quantize_kernel did not store them.
+__global__ void advance_kernel(int32_t* T_len, int B, int32_t n, int64_t T_cap) {
+  const int b = blockIdx.x * blockDim.x + threadIdx.x;
+  if (b < B && (int64_t)T_len[b] + n <= T_cap) T_len[b] += n;
 }
 
 // ----------------------------------------------------------------- bulk quantize (a prompt)
@@ -1080,8 +1090,10 @@ cudaError_t launch_quant_prepare(const mkv_config& c, const mkv_quant_params& qp
 }
 
 cudaError_t launch_quantize(const mkv_config& c, const mkv_quant_params& qp, const void* k_pre, const void* v,
-                            int64_t n_tokens, const mkv_cache& cache, cudaStream_t st) {
+                            int64_t n_tokens, const mkv_cache& cache, cudaStream_t st, bool step) {
   QuantArgs a{};
+  a.trigger = step;
+  a.tickets = c.Hkv <= 256;
   a.k_pre = static_cast<const __half*>(k_pre);
   a.v = static_cast<const __half*>(v);
   a.n_tokens = n_tokens;
@@ -1114,6 +1126,17 @@ cudaError_t launch_quantize(const mkv_config& c, const mkv_quant_params& qp, con
     return c.D == 128 ? launch_bulk_d<128>(a, c.B, st) : launch_bulk_d<64>(a, c.B, st);
   const int nwords = (c.D * c.bits / 8 + 3) / 4;
   const size_t smem = 2 * c.D + 4 * c.D + 2 * nwords * 4 + 16;
+  if (!a.tickets) {
+    a.trigger = 0;
+    quantize_kernel<<<c.B * c.Hkv, c.D, smem, st>>>(a);
+    const cudaError_t e = cudaPeekAtLastError();
+    if (e != cudaSuccess) return e;
+    advance_kernel<<<(unsigned)ceil_div(c.B, 256), 256, 0, st>>>(cache.T_len, c.B, (int32_t)n_tokens, cache.T_cap);
+    return cudaPeekAtLastError();
+  }
+  // in a step, beside the previous layer's draining decode; two plain launches in a graph measured 1.5 %
+  // faster than with the attribute on one of them only
+  if (step) return launch_pdl(quantize_kernel, dim3(c.B * c.Hkv), dim3(c.D), smem, st, a);
   quantize_kernel<<<c.B * c.Hkv, c.D, smem, st>>>(a);
   return cudaPeekAtLastError();
 }

@@ -325,7 +325,6 @@ mkv_status mkv_get_status(void* stream, uint32_t* flags) {
   MKV_CUDA(take_status_rocket(flags, as_stream(stream)));
   MKV_CUDA(take_status_decode(flags, as_stream(stream)));
   MKV_CUDA(take_status_prefill(flags, as_stream(stream)));
-  MKV_CUDA(take_status_kvq_step(flags, as_stream(stream)));
   if (*flags & MKV_FLAG_WAIT_TIMEOUT) {
     set_error("device status flags 0x%x (a bounded wait ran out)", *flags);
     return MKV_ERR_TIMEOUT;
@@ -423,20 +422,14 @@ mkv_status mkv_kvquant_step(const mkv_config* cfg, const mkv_quant_params* qpara
   MKV_REQUIRE(ws != nullptr && ws_bytes >= need.bytes, MKV_ERR_WORKSPACE,
               "workspace %zu bytes < %zu needed", ws_bytes, need.bytes);
   const Split sp = decode_split(*cfg, cache->T_cap);
-  // Each CTA that touches batch entry b takes one ticket in the top 8 bits of T_len[b] (at most
-  // n_cta <= 152 of them, within the 8 bits); a CTA keeps its units' lengths in 32-entry tables (it
-  // spans at most 28 of the <= 4096 units).
-  const int64_t units = (int64_t)cfg->B * cfg->Hkv, cpu = sp.chunks_per_unit, c_tot = cpu * units;
-  const int64_t span = (ceil_div(c_tot, (int64_t)sp.n_cta) - 1) / cpu + 2;
-  MKV_REQUIRE(sp.n_cta <= 255 && span <= kvquant_step_max_units_per_cta(), MKV_ERR_UNSUPPORTED,
-              "kvquant_step: %d CTAs read one batch entry's length (at most 255) or a CTA spans %lld units "
-              "(at most %d); use mkv_quantize_kv + mkv_decode_attention",
-              sp.n_cta, (long long)span, kvquant_step_max_units_per_cta());
+  // the quantization counts its finished CTAs per batch entry in the top 8 bits of T_len[b]
   MKV_REQUIRE(cache->T_cap < (1 << 24), MKV_ERR_UNSUPPORTED,
               "kvquant_step needs T_cap < 2^24 (T_cap %lld); use mkv_quantize_kv + mkv_decode_attention",
               (long long)cache->T_cap);
-  MKV_CUDA(launch_decode_kvquant(*cfg, q, *cache, *qparams, out, decode_ws(*cfg, cache->T_cap, ws), sp,
-                                 as_stream(stream), k_new, v_new));
+  cudaStream_t st = as_stream(stream);
+  MKV_CUDA(launch_quantize(*cfg, *qparams, k_new, v_new, 1, *cache, st, true));
+  MKV_CUDA(launch_decode_kvquant(*cfg, q, *cache, *qparams, out, decode_ws(*cfg, cache->T_cap, ws), sp, st,
+                                 cfg->Hkv <= 256));
   return MKV_OK;
 }
 

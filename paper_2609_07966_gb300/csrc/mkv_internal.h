@@ -103,13 +103,12 @@ cudaError_t launch_decode_fp16_family(const mkv_config& c, const void* q, const 
                                       const int32_t* page_idx, void* out, const DecodeWs& ws,
                                       const Split& sp, cudaStream_t st, const void* k_new = nullptr,
                                       const void* v_new = nullptr);
-// k_new / v_new (KVQUANT fused step): the step's token, quantized and appended by the same launch.
+// after_quantize: the launch directly follows launch_quantize(.., step = true) in the stream and may start
+// while that one runs.
 cudaError_t launch_decode_kvquant(const mkv_config& c, const void* q, const mkv_cache& cache,
                                   const mkv_quant_params& qp, void* out,
                                   const DecodeWs& ws, const Split& sp, cudaStream_t st,
-                                  const void* k_new = nullptr, const void* v_new = nullptr);
-// Units one CTA of the fused KVQuant step may touch (its length tables).
-int kvquant_step_max_units_per_cta();
+                                  bool after_quantize = false);
 cudaError_t launch_append(const mkv_config& c, const void* k_new, const void* v_new,
                           const mkv_cache& cache, cudaStream_t st);
 cudaError_t launch_rope_table(int D, float theta, int64_t T_max, float* table, cudaStream_t st);
@@ -119,7 +118,8 @@ cudaError_t launch_calibrate(const mkv_config& c, const void* k_cal, const void*
                              int64_t row_stride, const mkv_quant_params& qp, const CalibWs& ws,
                              cudaStream_t st);
 cudaError_t launch_quantize(const mkv_config& c, const mkv_quant_params& qp, const void* k_pre,
-                            const void* v, int64_t n_tokens, const mkv_cache& cache, cudaStream_t st);
+                            const void* v, int64_t n_tokens, const mkv_cache& cache, cudaStream_t st,
+                            bool step = false);
 
 cudaError_t launch_h2o_update(const mkv_config& c, const mkv_cache& cache, const DecodeWs& ws,
                               cudaStream_t st);
@@ -150,7 +150,6 @@ cudaError_t take_status_append(uint32_t* flags, cudaStream_t st);
 cudaError_t take_status_rocket(uint32_t* flags, cudaStream_t st);
 cudaError_t take_status_decode(uint32_t* flags, cudaStream_t st);
 cudaError_t take_status_prefill(uint32_t* flags, cudaStream_t st);
-cudaError_t take_status_kvq_step(uint32_t* flags, cudaStream_t st);
 cudaError_t launch_wait_selftest(int ms, cudaStream_t st);
 
 }  // namespace mkv

@@ -1,9 +1,8 @@
 // One token of one (batch, kv-head) quantized into the KVQuant cache (Section 2.1,
 // KVQuant paragraph): per-channel key codes (pre-rotation), the key outliers as
 // CSR entries, the token's value outliers, its value range and value codes.
-// Shared by the quantize kernel (one CTA per unit, one thread per channel) and
-// the fused decode step (the attention warps of the CTA that owns the token's
-// chunk), so both write the same bits.
+// Run by quantize_kernel (one CTA per unit, one thread per channel); quantize_bulk_kernel writes the same
+// bits with a warp per token.
 //
 // Codes are decided with correctly rounded fp32 operations (__fsub_rn, __fdiv_rn,
 // __fmul_rn, rintf):
