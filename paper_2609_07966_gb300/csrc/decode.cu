@@ -490,7 +490,8 @@ extern "C" mkv_status mkv_decode_attention_noalloc(const mkv_config* cfg, const 
   using namespace mkv;
   const mkv_status st0 = check_fp16_decode_args(cfg, cache, q, out);
   if (st0 != MKV_OK) return st0;
-  const DecodeWs need = decode_ws(*cfg, cache->T_cap, nullptr);
+  const Split sp = decode_split(*cfg, cache->T_cap);
+  const DecodeWs need = decode_ws(*cfg, cache->T_cap, sp, nullptr);
   if (need.bytes > kNoAllocScratchBytes) {
     set_error("this call needs %zu bytes of scratch; the built-in array holds %zu (use mkv_decode_attention "
               "with a workspace)", need.bytes, kNoAllocScratchBytes);
@@ -502,8 +503,7 @@ extern "C" mkv_status mkv_decode_attention_noalloc(const mkv_config* cfg, const 
     set_error("cudaGetSymbolAddress of the built-in scratch: %s", cudaGetErrorString(e));
     return MKV_ERR_CUDA;
   }
-  const DecodeWs w = decode_ws(*cfg, cache->T_cap, scratch);
-  const Split sp = decode_split(*cfg, cache->T_cap);
+  const DecodeWs w = decode_ws(*cfg, cache->T_cap, sp, scratch);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   e = launch_decode_fp16_family(*cfg, q, *cache, nullptr, out, w, sp, st);
   if (e != cudaSuccess) {

@@ -357,7 +357,7 @@ __global__ void __launch_bounds__(kThr, 1) decode_kvq_kernel(const KvqArgs a) {
       }
     }
     __syncthreads();                   // the stage buffers now serve as the merge's scratch
-    merge_if_last<D, kThr>(a.merge, bh, b, kvh, reinterpret_cast<float*>(stg), Lay::NS * Lay::STAGE / 4, parts);
+    merge_if_last_lean<D, kThr>(a.merge, bh, b, kvh, reinterpret_cast<float*>(stg), Lay::NS * Lay::STAGE / 4, parts);
     __syncthreads();                   // before the next segment's copies into the stages
   };
 

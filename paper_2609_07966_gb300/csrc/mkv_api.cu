@@ -34,21 +34,42 @@ Split decode_split(const mkv_config& c, int64_t T_cap) {
   // kernel one.  Pick the split count that minimises (waves of CTAs) x
   // (chunks per CTA), i.e. the time of the busiest SM; among equals prefer
   // fewer splits (smaller partials).
-  const int64_t slots = (c.method == MKV_KVQUANT ? 1 : 2) * kNumSMs;
+  const int64_t slots = 2 * kNumSMs;
   int64_t best_n = 1, best_cost = INT64_MAX;
-  for (int64_t n = 1; n <= std::min<int64_t>(chunks, 1024); ++n) {
-    const int64_t cps = ceil_div(chunks, n);
-    if (ceil_div(chunks, cps) != n) continue;      // n is not the split count of any cps
-    // + 6: a CTA's fixed cost (query and table loads, pipeline fill and drain, merge) in chunk
-    // units, fitted to measured split sweeps of the FP16 and KVQuant kernels
-    const int64_t cost = ceil_div(units * n, slots) * (cps + 6);
-    if (cost < best_cost) {
-      best_cost = cost;
-      best_n = n;
+  if (c.method != MKV_KVQUANT) {
+    // the split counts that some number of chunks per split has, most splits first
+    for (int64_t n = std::min<int64_t>(chunks, 1024); n >= 1;) {
+      const int64_t cps = ceil_div(chunks, n);
+      n = ceil_div(chunks, cps);
+      // + 6: a CTA's fixed cost (query and table loads, pipeline fill and drain, merge) in chunk
+      // units, fitted to measured split sweeps of the FP16 kernels
+      const int64_t cost = ceil_div(units * n, slots) * (cps + 6);
+      if (cost <= best_cost) {
+        best_cost = cost;
+        best_n = n;
+      }
+      --n;
     }
   }
   s.chunks_per_split = (int)ceil_div(chunks, best_n);
-  s.n_split = (int)ceil_div(chunks, s.chunks_per_split);
+  s.n_slots = s.n_split = (int)ceil_div(chunks, s.chunks_per_split);
+  if (c.method != MKV_KVQUANT) {
+    // That is the most splits (the workspace and the step's ticket limit count it).  Within it, a split
+    // also costs the merge, about a quarter of a chunk: batch 1, 32/8 heads, T = 4096: 33 splits of 2 chunks 12.6
+    // us a step, 17 of 4 9.9 us; T = 2000: 32 of 1 11.8 us, 11 of 3 8.8 us; with many units nothing changes.
+    int64_t best100 = INT64_MAX, cps_best = s.chunks_per_split;
+    for (int64_t cps = s.chunks_per_split; cps <= chunks; ++cps) {
+      const int64_t n = ceil_div(chunks, cps);
+      const int64_t cost100 = 100 * ceil_div(units * n, slots) * (cps + 6) + 25 * n;
+      if (cost100 < best100) {
+        best100 = cost100;
+        cps_best = cps;
+      }
+      if (100 * (cps + 6) > best100 || (c.method == MKV_ROCKET && (cps + 1) * (kChunk / kPage) + 1 > 1024)) break;
+    }
+    s.chunks_per_split = (int)cps_best;
+    s.n_split = (int)ceil_div(chunks, cps_best);
+  }
   if (c.method == MKV_KVQUANT) {
     // one CTA per SM, each over an equal range of all units' chunks (at most a few units per
     // CTA); a unit's partial slots are the CTAs that cover part of it
@@ -60,14 +81,13 @@ Split decode_split(const mkv_config& c, int64_t T_cap) {
       const int64_t n = cta_of_chunk((u + 1) * chunks - 1, c_tot, s.n_cta) - cta_of_chunk(u * chunks, c_tot, s.n_cta) + 1;
       slots_max = std::max(slots_max, n);
     }
-    s.n_split = (int)slots_max;
+    s.n_slots = s.n_split = (int)slots_max;
     s.chunks_per_split = (int)chunks;
   }
   return s;
 }
 
-DecodeWs decode_ws(const mkv_config& c, int64_t T_cap, void* base) {
-  const Split sp = decode_split(c, T_cap);
+DecodeWs decode_ws(const mkv_config& c, int64_t T_cap, const Split& sp, void* base) {
   const size_t hq = (size_t)c.B * c.Hq;
   uint8_t* p = static_cast<uint8_t*>(base);
   size_t off = kCounterBytes;
@@ -77,9 +97,9 @@ DecodeWs decode_ws(const mkv_config& c, int64_t T_cap, void* base) {
     off += align256(bytes);
     return r;
   };
-  w.part_m = take(hq * sp.n_split * 4);
-  w.part_l = take(hq * sp.n_split * 4);
-  w.part_o = take(hq * sp.n_split * c.D * 4);
+  w.part_m = take(hq * sp.n_slots * 4);
+  w.part_l = take(hq * sp.n_slots * 4);
+  w.part_o = take(hq * sp.n_slots * c.D * 4);
   w.counters = base ? static_cast<int*>(base) : nullptr;
   if (c.method == MKV_H2O) {
     w.logits = take((size_t)c.B * c.Hkv * T_cap * (c.Hq / c.Hkv) * 4);
@@ -242,7 +262,7 @@ mkv_status check_qparams(const mkv_config* c, const mkv_quant_params* p, bool ne
   } while (0)
 
 size_t workspace_bytes(const mkv_config* c, int64_t T_cap) {
-  size_t b = decode_ws(*c, T_cap, nullptr).bytes;
+  size_t b = decode_ws(*c, T_cap, decode_split(*c, T_cap), nullptr).bytes;
   if (c->method == MKV_H2O || c->method == MKV_ROCKET) b = std::max(b, prefill_ws(*c, T_cap, nullptr).bytes);
   if (c->method == MKV_KVQUANT) b = std::max(b, calib_ws(*c, std::min<int64_t>(T_cap, 4096), nullptr).bytes);
   return b;
@@ -364,11 +384,11 @@ mkv_status mkv_decode_attention(const mkv_config* cfg, const void* q, const mkv_
                 "KVQUANT decode indexes key outliers and tokens with 32 bits (k_out_cap %lld, T_cap %lld)",
                 (long long)cache->k_out_cap, (long long)cache->T_cap);
   }
-  const DecodeWs need = decode_ws(*cfg, cache->T_cap, nullptr);
+  const Split sp = decode_split(*cfg, cache->T_cap);
+  const DecodeWs need = decode_ws(*cfg, cache->T_cap, sp, nullptr);
   MKV_REQUIRE(ws != nullptr && ws_bytes >= need.bytes, MKV_ERR_WORKSPACE,
               "workspace %zu bytes < %zu needed", ws_bytes, need.bytes);
-  const DecodeWs w = decode_ws(*cfg, cache->T_cap, ws);
-  const Split sp = decode_split(*cfg, cache->T_cap);
+  const DecodeWs w = decode_ws(*cfg, cache->T_cap, sp, ws);
   MKV_REQUIRE(cfg->method != MKV_ROCKET || (int64_t)sp.chunks_per_split * (kChunk / kPage) + 1 <= 1024,
               MKV_ERR_UNSUPPORTED, "topk_pages too large for one decode split");
   cudaStream_t st = as_stream(stream);
@@ -389,16 +409,16 @@ mkv_status mkv_decode_step(const mkv_config* cfg, const void* q, const void* k_n
   MKV_REQUIRE(q && out && k_new && v_new, MKV_ERR_INVALID_ARG, "q/out/k_new/v_new NULL");
   MKV_REQUIRE(((uintptr_t)k_new | (uintptr_t)v_new) % 16 == 0, MKV_ERR_INVALID_ARG,
               "k_new/v_new must be 16-byte aligned (the step reads them in 16-byte pieces)");
-  const DecodeWs need = decode_ws(*cfg, cache->T_cap, nullptr);
+  const Split sp = decode_split(*cfg, cache->T_cap);
+  const DecodeWs need = decode_ws(*cfg, cache->T_cap, sp, nullptr);
   MKV_REQUIRE(ws != nullptr && ws_bytes >= need.bytes, MKV_ERR_WORKSPACE,
               "workspace %zu bytes < %zu needed", ws_bytes, need.bytes);
-  const Split sp = decode_split(*cfg, cache->T_cap);
   // the launch counts its finished CTAs per batch entry (Hkv x splits) in the top 8 bits of T_len[b]
-  MKV_REQUIRE(cache->T_cap < (1 << 24) && (int64_t)cfg->Hkv * sp.n_split <= 255, MKV_ERR_UNSUPPORTED,
+  MKV_REQUIRE(cache->T_cap < (1 << 24) && (int64_t)cfg->Hkv * sp.n_slots <= 255, MKV_ERR_UNSUPPORTED,
               "decode_step needs T_cap < 2^24 and Hkv * splits <= 255 (T_cap %lld, Hkv %d, splits %d); use "
               "mkv_append_kv + mkv_decode_attention",
-              (long long)cache->T_cap, cfg->Hkv, sp.n_split);
-  MKV_CUDA(launch_decode_fp16_family(*cfg, q, *cache, nullptr, out, decode_ws(*cfg, cache->T_cap, ws), sp,
+              (long long)cache->T_cap, cfg->Hkv, sp.n_slots);
+  MKV_CUDA(launch_decode_fp16_family(*cfg, q, *cache, nullptr, out, decode_ws(*cfg, cache->T_cap, sp, ws), sp,
                                      as_stream(stream), k_new, v_new));
   return MKV_OK;
 }
@@ -418,17 +438,17 @@ mkv_status mkv_kvquant_step(const mkv_config* cfg, const mkv_quant_params* qpara
   MKV_REQUIRE(cache->k_out_cap <= INT32_MAX && cache->T_cap < INT32_MAX, MKV_ERR_UNSUPPORTED,
               "KVQUANT decode indexes key outliers and tokens with 32 bits (k_out_cap %lld, T_cap %lld)",
               (long long)cache->k_out_cap, (long long)cache->T_cap);
-  const DecodeWs need = decode_ws(*cfg, cache->T_cap, nullptr);
+  const Split sp = decode_split(*cfg, cache->T_cap);
+  const DecodeWs need = decode_ws(*cfg, cache->T_cap, sp, nullptr);
   MKV_REQUIRE(ws != nullptr && ws_bytes >= need.bytes, MKV_ERR_WORKSPACE,
               "workspace %zu bytes < %zu needed", ws_bytes, need.bytes);
-  const Split sp = decode_split(*cfg, cache->T_cap);
   // the quantization counts its finished CTAs per batch entry in the top 8 bits of T_len[b]
   MKV_REQUIRE(cache->T_cap < (1 << 24), MKV_ERR_UNSUPPORTED,
               "kvquant_step needs T_cap < 2^24 (T_cap %lld); use mkv_quantize_kv + mkv_decode_attention",
               (long long)cache->T_cap);
   cudaStream_t st = as_stream(stream);
   MKV_CUDA(launch_quantize(*cfg, *qparams, k_new, v_new, 1, *cache, st, true));
-  MKV_CUDA(launch_decode_kvquant(*cfg, q, *cache, *qparams, out, decode_ws(*cfg, cache->T_cap, ws), sp, st,
+  MKV_CUDA(launch_decode_kvquant(*cfg, q, *cache, *qparams, out, decode_ws(*cfg, cache->T_cap, sp, ws), sp, st,
                                  cfg->Hkv <= 256));
   return MKV_OK;
 }
@@ -495,10 +515,11 @@ mkv_status mkv_h2o_update(const mkv_config* cfg, mkv_cache* cache, void* ws, siz
   MKV_TRY(check_config(cfg));
   MKV_REQUIRE(cfg->method == MKV_H2O, MKV_ERR_INVALID_ARG, "h2o_update is for H2O");
   MKV_TRY(check_cache(cfg, cache));
-  const DecodeWs need = decode_ws(*cfg, cache->T_cap, nullptr);
+  const Split sp = decode_split(*cfg, cache->T_cap);
+  const DecodeWs need = decode_ws(*cfg, cache->T_cap, sp, nullptr);
   MKV_REQUIRE(ws != nullptr && ws_bytes >= need.bytes, MKV_ERR_WORKSPACE,
               "workspace %zu bytes < %zu needed", ws_bytes, need.bytes);
-  MKV_CUDA(launch_h2o_update(*cfg, *cache, decode_ws(*cfg, cache->T_cap, ws), as_stream(stream)));
+  MKV_CUDA(launch_h2o_update(*cfg, *cache, decode_ws(*cfg, cache->T_cap, sp, ws), as_stream(stream)));
   return MKV_OK;
 }
 

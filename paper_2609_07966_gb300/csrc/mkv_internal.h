@@ -29,7 +29,8 @@ inline size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 // Work split of a decode call: `n_split` CTAs per (batch, kv-head), each over
 // `chunks_per_split` chunks of kChunk virtual tokens (KVQuant: a balanced range per CTA).
 struct Split {
-  int n_split;           // partial slots per (batch, kv-head)
+  int n_split;           // splits (KVQuant: partial slots) per (batch, kv-head)
+  int n_slots;           // most splits the call's workspace and limits allow for (>= n_split)
   int chunks_per_split;
   int64_t v_tokens;      // virtual tokens per (batch, kv-head)
   // KVQuant: one CTA per SM over the concatenated chunks of all (batch, kv-head) units; CTA i
@@ -55,7 +56,7 @@ struct DecodeWs {
   int* counters;   // [B][Hkv] split tickets; zero between calls
   size_t bytes;
 };
-DecodeWs decode_ws(const mkv_config& c, int64_t T_cap, void* base);
+DecodeWs decode_ws(const mkv_config& c, int64_t T_cap, const Split& sp, void* base);
 
 // Prefill workspace (H2O prefill, SnapKV compression): scores and selection.
 struct PrefillWs {
