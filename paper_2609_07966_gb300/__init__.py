@@ -144,10 +144,17 @@ def config(method: int, B: int, Hq: int, Hkv: int, D: int, **kw) -> mkv_config:
 
 
 def _stream(stream):
-    if stream is None:
-        import torch
+    """The cudaStream_t of `stream`, or of torch's current stream on its current device (None).
+
+    The current stream is asked for as a handle: 0.4 us a call, 3.0 through torch.cuda.current_stream(), which
+    makes a Python object of it (a whole mkv_decode_step call of a small model: 4.1 us, 7.6 with that).
+    """
+    if stream is not None:
+        return int(stream)
+    import torch
+    if not torch.cuda.is_initialized():
         return torch.cuda.current_stream().cuda_stream
-    return int(stream)
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def mkv_workspace_size(cfg: mkv_config, T_cap: int) -> int:
