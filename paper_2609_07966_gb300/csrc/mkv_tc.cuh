@@ -136,7 +136,15 @@ __device__ __forceinline__ void tc_wait_ld_regs(uint32_t (&r)[32]) {
                : "memory");
 }
 
-// 64 consecutive fp32 columns (four loads in flight, then the wait)
+// 32 and 64 consecutive fp32 columns (two, four loads in flight, then the wait)
+__device__ __forceinline__ void tc_ld32(uint32_t taddr, float (&v)[32]) {
+  uint32_t r[32];
+  tc_ld16_issue(taddr, *reinterpret_cast<uint32_t(*)[16]>(&r[0]));
+  tc_ld16_issue(taddr + 16, *reinterpret_cast<uint32_t(*)[16]>(&r[16]));
+  tc_wait_ld_regs(r);
+#pragma unroll
+  for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
+}
 __device__ __forceinline__ void tc_ld64(uint32_t taddr, float (&v)[64]) {
   uint32_t r0[32], r1[32];
   tc_ld16_issue(taddr, *reinterpret_cast<uint32_t(*)[16]>(&r0[0]));

@@ -7,28 +7,29 @@
 //
 // Two passes on the 5th-generation tensor cores (tcgen05.mma kind::f16: fp16 operands, fp32
 // accumulator in tensor memory), each a stream of 128 x N x D tile products with a softmax epilogue:
-//   pass 1 (rows): a CTA holds 128 query rows (the group's G heads, 128 / G rows each) and streams
-//           256-key tiles (N = 256: one MMA instruction and one barrier round trip per 256 keys); it
-//           keeps per row the running max m and sum l of 2^(s - m) over the causal keys.  When the
+//   pass 1 (rows): a CTA holds one or two blocks of 128 query rows (the group's G heads, 128 / G rows each)
+//           and streams 256-key tiles (N = 256: one MMA instruction and one barrier round trip per 256
+//           keys); it keeps per row the running max m and sum l of 2^(s - m) over the causal keys.  When the
 //           rows are few (an observation window) the key range is split across CTAs; a small kernel
 //           merges the splits into (-m, 1 / l) per row, laid out in the order of pass 2's query blocks;
-//   pass 2 (columns): a CTA holds 128 keys and streams the 128-row query blocks that can see them
-//           (N = 128, four accumulator buffers: its epilogue is the heavier one), summing
-//           2^(s - m_i) / l_i over the rows with p_i >= j for each key j;
+//   pass 2 (columns): a CTA holds 256 keys, or 128 when there are few, and streams the 128-row query
+//           blocks that can see them, summing 2^(s - m_i) / l_i over the rows with p_i >= j for each key j;
 //   pass 2 over one query block (colsum_window_kernel): when the window's rows fit one block, a
 //           CTA holds that block and streams a run of 128-key tiles instead.
 // The held operand is the MMA's A (M = 128 lanes of the accumulator), a streamed tile its B (the
-// window kernel swaps them).  Each CTA is warp-specialised, one per SM (all 512 tensor-memory
+// 256-key and the window kernel swap them).  Each CTA is warp-specialised, one per SM (all 512 tensor-memory
 // columns):
 //   warp 0 (one thread) loads operand tiles by TMA (tensor maps with the 128-byte swizzle, the
 //           K-major layout the MMA reads) into a ring of stages, and in pass 2 each query block's
 //           128 row statistics by a bulk copy beside it;
 //   warp 1 (one thread) issues the D / 16 MMAs of tile t into accumulator buffer t % (buffers),
 //           then commits to the stage's and the buffer's mbarriers;
-//   warps 2..17 read finished accumulators in two groups of eight: group g takes the tiles
-//           t = g mod 2, so the groups work a tile apart and one group's exponentials overlap the
+//   warps 2..17 read finished accumulators in two groups of eight: group g takes the products
+//           t = g mod 2, so the groups work a product apart and one group's exponentials overlap the
 //           other's loads and reductions; warp w reads lanes 32 (w % 4) .. + 31 (the lane quarter it
-//           may access) and one half of the tile's columns, 64 at a time.
+//           may access) and one half of the product's columns, 64 at a time (the 256-key kernel: all
+//           sixteen take every product, a quarter of its columns each).  A buffer is given back as soon as
+//           it is read, before the exponentials of what was read.
 // Loads, products and epilogues of different tiles overlap; nothing in the tile loop waits on a
 // CTA-wide barrier.  Every wait is bounded (1 s of the GPU's global timer): on a timeout the role
 // raises MKV_FLAG_WAIT_TIMEOUT and sets a flag that ends the other roles' waits; the CTA then waits
@@ -90,7 +91,7 @@ struct ScoreArgs {
   float* score2;        // one query block: the sums of its second 64 rows (or null: added onto a zeroed score)
 };
 
-template <int D, int TN>
+template <int D, int TN, int HELD = 1>
 struct Layout {
   using C = Tiling<TN>;
   static constexpr int ATOM_A = kTM * 128;                // 128 rows x 64 fp16: one swizzle-atom column
@@ -98,7 +99,7 @@ struct Layout {
   static constexpr int TILE_A = (D / 64) * ATOM_A;
   static constexpr int TILE_B = (D / 64) * ATOM_B;
   static constexpr int A_OFF = 0;
-  static constexpr int B_OFF = TILE_A;                    // [kS] streamed tiles
+  static constexpr int B_OFF = HELD * TILE_A;             // [kS] streamed tiles
   static constexpr int ST_OFF = B_OFF + C::kS * TILE_B;   // [kS][kBlocks] pass 2: the query blocks' statistics
   static constexpr int MRG_OFF = ST_OFF + C::kS * C::kBlocks * kStatBytes;   // [4][128] (group, half) partials
   static constexpr int CTL_OFF = MRG_OFF + 4 * kTM * 8;
@@ -203,15 +204,16 @@ __device__ __forceinline__ void cta_teardown(Ctl<TN>* ctl, uint32_t tbase) {
   if ((threadIdx.x >> 5) == 0) tc_dealloc(tbase, C::kNB * TN);
 }
 
-// The three roles over `ntiles` streamed tiles.  issue_a(bar) loads the held operand;
-// issue_b(t, s, bar) loads tile t into stage s; epi(t, col, s) reads the thread's half of tile t's
-// accumulator (kHalf columns from tensor-memory address col, lane 0) and, with kStats, the
-// statistics of stage s.  With kStreamA the streamed tile is the MMA's A operand and the held one its
-// B (the accumulator's lanes then follow the streamed rows).
-template <int D, int TN, bool kStats, bool kStreamA = false, typename IssueA, typename IssueB, typename Epi>
+// The three roles over `ntiles` streamed tiles.  issue_a(bar) loads the held operand, or both (kHeld = 2:
+// each tile then gives two products, the second held operand's after the first's, one per epilogue
+// group); issue_b(t, s, bar) loads tile t into stage s; epi(t, col, s, release) reads the thread's half of a
+// product (kHalf columns from tensor-memory address col, lane 0), calls release() once that is read and,
+// with kStats, uses the statistics of stage s.  With kStreamA the streamed tile is the MMA's A operand and
+// the held one its B (the accumulator's lanes then follow the streamed rows).
+template <int D, int TN, bool kStats, bool kStreamA = false, int kHeld = 1, typename IssueA, typename IssueB, typename Epi>
 __device__ __forceinline__ void run_roles(uint8_t* sm, Ctl<TN>* ctl, uint32_t tbase, int ntiles, IssueA issue_a,
                                           IssueB issue_b, Epi epi) {
-  using L = Layout<D, TN>;
+  using L = Layout<D, TN, kHeld>;
   using C = Tiling<TN>;
   constexpr int kS = C::kS, kNB = C::kNB, kHalf = C::kHalf;
   volatile int* fail = &ctl->fail;
@@ -236,18 +238,24 @@ __device__ __forceinline__ void run_roles(uint8_t* sm, Ctl<TN>* ctl, uint32_t tb
       const uint64_t b_desc = tc_desc_sw128(smem_addr(sm + L::B_OFF));
       if (role_wait(&ctl->abar, 0, fail)) {
         for (int t = 0; t < ntiles; ++t) {
-          const int s = t % kS, bf = t % kNB, u = t / kNB;
+          const int s = t % kS;
           if (!role_wait(&ctl->full[s], (uint32_t)((t / kS) & 1), fail)) break;
-          if (u > 0 && !role_wait(&ctl->tempty[bf], (uint32_t)((u - 1) & 1), fail)) break;
-          tc_fence_after();
+          bool ok = true;
           const uint64_t stage = b_desc + (uint64_t)((s * L::TILE_B) >> 4);
-          if (kStreamA)
-            issue_tile<D, TN>(tbase + (uint32_t)(bf * TN), stage, a_desc);
-          else
-            issue_tile<D, TN>(tbase + (uint32_t)(bf * TN), a_desc, stage);
-          tc_commit(&ctl->empty[s]);
-          tc_commit(&ctl->tfull[bf]);
-          ctl->mma_issued = t + 1;
+          for (int h = 0; h < kHeld; ++h) {   // a product per held operand
+            const int x = t * kHeld + h, bf = x % kNB, u = x / kNB;
+            if (u > 0) ok = role_wait(&ctl->tempty[bf], (uint32_t)((u - 1) & 1), fail);
+            if (!ok) break;
+            tc_fence_after();
+            if (kStreamA)
+              issue_tile<D, TN>(tbase + (uint32_t)(bf * TN), stage, a_desc);
+            else
+              issue_tile<D, TN>(tbase + (uint32_t)(bf * TN), a_desc + (uint64_t)((h * L::TILE_A) >> 4), stage);
+            if (h == kHeld - 1) tc_commit(&ctl->empty[s]);
+            tc_commit(&ctl->tfull[bf]);
+            ctl->mma_issued = x + 1;
+          }
+          if (!ok) break;
         }
       }
     }
@@ -256,45 +264,52 @@ __device__ __forceinline__ void run_roles(uint8_t* sm, Ctl<TN>* ctl, uint32_t tb
     // the held operand's phase: what came with it (statistics held beside it) is visible after it
     const bool held = role_wait(&ctl->abar, 0, fail);
     if (!__all_sync(0xffffffffu, held)) return;
-    for (int t = grp; t < ntiles; t += 2) {
-      const int s = t % kS, bf = t % kNB;
-      bool ok = role_wait(&ctl->tfull[bf], (uint32_t)((t / kNB) & 1), fail);
+    for (int x = grp; x < kHeld * ntiles; x += 2) {   // (two held operands: one per group)
+      const int t = x / kHeld, s = t % kS, bf = x % kNB;
+      bool ok = role_wait(&ctl->tfull[bf], (uint32_t)((x / kNB) & 1), fail);
       // the statistics came with the stage's operand: their copy completed that phase of full[s]
       if (kStats) ok = ok && role_wait(&ctl->full[s], (uint32_t)((t / kS) & 1), fail);
       if (!__all_sync(0xffffffffu, ok)) break;
       tc_fence_after();
-      epi(t, tbase + (uint32_t)(bf * TN + half * kHalf), s);
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) {
-        tc_mbar_arrive(&ctl->tempty[bf]);
-        if (kStats) tc_mbar_arrive(&ctl->sempty[s]);
+      epi(t, tbase + (uint32_t)(bf * TN + half * kHalf), s, [&]() {
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) tc_mbar_arrive(&ctl->tempty[bf]);
+      });
+      if (kStats) {
+        __syncwarp();
+        if (lane == 0) tc_mbar_arrive(&ctl->sempty[s]);
       }
     }
   }
 }
 
 // ---------------------------------------------------------------- pass 1
-template <int D>
+// HELD = 2: two row blocks per CTA, a key tile read once for both.  Bound by L2 reads and the products' waits
+// before the exponentials: 32/8 heads, D 128, batch 16, T = 512 (1024 block pairs): both passes 132.9 us with
+// one block per CTA, 112.3 with two; batch 4, T = 2048: 228 and 204.  (Giving the buffers back early: batch 2,
+// T = 16384 3.85 -> 3.65 ms.)
+template <int D, int HELD>
 __global__ void __launch_bounds__(kThr, 1)
     rowstats_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant__ CUtensorMap kmap,
                        const ScoreArgs a) {
   constexpr int kTN = kTN1, kHalf = Tiling<kTN1>::kHalf;
-  using L = Layout<D, kTN1>;
+  using L = Layout<D, kTN1, HELD>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* sm = align1024(smem_raw);
   Ctl<kTN1>* ctl = reinterpret_cast<Ctl<kTN1>*>(sm + L::CTL_OFF);
-  const int ks = blockIdx.x;
-  const int rb = a.rowblocks - 1 - (int)blockIdx.y;      // the row blocks with the most keys first
-  const int bh = (int)blockIdx.z;
+  const int ks = HELD == 2 ? 0 : blockIdx.x;
+  const int rb0 = (a.rowblocks - 1) / HELD * HELD - HELD * (int)blockIdx.y;   // the blocks with the most keys first
+  const int bh = HELD == 2 ? (int)blockIdx.x : (int)blockIdx.z;
   const int b = bh / a.Hkv, kvh = bh % a.Hkv;
   const int warp = threadIdx.x >> 5;
   const int lq = warp & 3, cq = (warp - 2) >> 2;         // (epilogue warps) lane quarter; group x half
   const int hf = cq & 1;                                 // column half of the tile
   const int lr = lq * 32 + (threadIdx.x & 31);           // accumulator lane = query row of the block
 
-  // the block's last valid row bounds its causal key range
-  const int64_t row_hi = std::min<int64_t>((int64_t)rb * a.rpb + a.rpb, a.R);   // exclusive
+  const int rb = rb0 + (HELD == 2 ? cq >> 1 : 0);        // (epilogue warps) the group's row block
+  // the last valid row bounds the causal key range
+  const int64_t row_hi = std::min<int64_t>((int64_t)(rb0 + HELD) * a.rpb, a.R);   // exclusive
   const int64_t k_begin = (int64_t)ks * a.tiles_per_split * kTN;
   const int64_t k_end = std::min<int64_t>(std::min<int64_t>(k_begin + (int64_t)a.tiles_per_split * kTN, a.T),
                                           a.pos0 + row_hi);
@@ -304,12 +319,13 @@ __global__ void __launch_bounds__(kThr, 1)
 
   const uint32_t tbase = cta_setup(ctl);
   float m_run = -INFINITY, l_run = 0.f;
-  run_roles<D, kTN1, false>(
+  run_roles<D, kTN1, false, false, HELD>(
       sm, ctl, tbase, ntiles,
       [&](uint64_t* bar) {                // one box of G heads x rpb rows: head g's rows are tile rows g rpb ..
-        tc_mbar_expect_tx(bar, L::TILE_A);
-        for (int at = 0; at < D / 64; ++at)
-          tma_load_4d(sm + L::A_OFF + at * L::ATOM_A, &qmap, at * 64, rb * a.rpb, kvh * a.G, b, bar);
+        tc_mbar_expect_tx(bar, HELD * L::TILE_A);
+        for (int h = 0; h < HELD; ++h)
+          for (int at = 0; at < D / 64; ++at)
+            tma_load_4d(sm + L::A_OFF + h * L::TILE_A + at * L::ATOM_A, &qmap, at * 64, (rb0 + h) * a.rpb, kvh * a.G, b, bar);
       },
       [&](int t, int s, uint64_t* bar) {
         tc_mbar_expect_tx(bar, L::TILE_B);
@@ -317,12 +333,13 @@ __global__ void __launch_bounds__(kThr, 1)
           tma_load_4d(sm + L::B_OFF + s * L::TILE_B + at * L::ATOM_B, &kmap, at * 64,
                       (int)(k_begin + (int64_t)t * kTN), kvh, b, bar);
       },
-      [&](int t, uint32_t col, int) {
+      [&](int t, uint32_t col, int, auto release) {
 #pragma unroll 1
         for (int ch = 0; ch < kHalf / 64; ++ch) {
           const int64_t jc = k_begin + (int64_t)t * kTN + hf * kHalf + ch * 64;
           float v[64];
           tc_ld64(col + ((uint32_t)(lq * 32) << 16) + (uint32_t)(ch * 64), v);
+          if (ch == kHalf / 64 - 1) release();
           if (jc + 63 > lim) {            // keys past the row's causal limit (or the range) drop out
 #pragma unroll
             for (int e = 0; e < 64; ++e) v[e] = jc + e <= lim ? v[e] : -INFINITY;
@@ -347,19 +364,20 @@ __global__ void __launch_bounds__(kThr, 1)
           }
         }
       });
-  // the (group, half) partials of each row merged into this split's (m, l)
+  // the partials of each row (from the column halves; one held operand: and the groups) merged into this split's (m, l)
   float2* mrg = reinterpret_cast<float2*>(sm + L::MRG_OFF);
   if (warp >= 2) mrg[cq * kTM + lr] = make_float2(m_run, l_run);
   __syncthreads();
-  if (warp >= 2 && cq == 0) {
+  constexpr int NP = 4 / HELD;
+  if (warp >= 2 && cq % NP == 0 && rb < a.rowblocks) {
     float M = -INFINITY;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) M = fmaxf(M, mrg[q * kTM + lr].x);
+    for (int q = 0; q < NP; ++q) M = fmaxf(M, mrg[(cq + q) * kTM + lr].x);
     float l = 0.f;
     if (M != -INFINITY) {
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const float2 o = mrg[q * kTM + lr];
+      for (int q = 0; q < NP; ++q) {
+        const float2 o = mrg[(cq + q) * kTM + lr];
         l += o.y * ex2_approx(o.x - M);
       }
     }
@@ -437,7 +455,7 @@ __global__ void __launch_bounds__(kThr, 1)
                     stats + (int64_t)(rb + h) * a.n_ksplit * kTM, kStatBytes, bar);
         }
       },
-      [&](int t, uint32_t col, int s) {
+      [&](int t, uint32_t col, int s, auto release) {
         const uint64_t sc2 = pk2(a.scale_log2, a.scale_log2);
         uint64_t sp2[2] = {0ull, 0ull};
 #pragma unroll 1
@@ -445,13 +463,13 @@ __global__ void __launch_bounds__(kThr, 1)
           const int c0 = hf * C::kHalf + ch * 64;   // the chunk's first column of the tile
           const int h = c0 / kBlk, cin = c0 % kBlk;   // its query block and first column in the block
           const int rb = rb_begin + C::kBlocks * t + h;
-          if (rb >= a.rowblocks) break;           // a block past the query rows (warp-uniform)
           const int64_t i0 = (int64_t)rb * a.rpb;   // row index of the block's first row per head
           // row pair p's statistics {-m, -m', 1/l, 1/l'}
           const float4* s4 =
               reinterpret_cast<const float4*>(sm + L::ST_OFF + (s * C::kBlocks + h) * kStatBytes) + cin / 2;
           float v[64];
           tc_ld64(col + ((uint32_t)(lq * 32) << 16) + (uint32_t)(ch * 64), v);
+          release();
           if (i0 >= j0 + kBlk - 1 - a.pos0) {   // every row sees every key of the CTA: two rows per instruction
 #pragma unroll
             for (int q = 0; q < 32; ++q) {
@@ -481,6 +499,193 @@ __global__ void __launch_bounds__(kThr, 1)
   if (warp >= 2 && cq == 0 && j0 + lr < a.T)
     a.score[(int64_t)bh * a.T + j0 + lr] = (mrg[lr] + mrg[kTM + lr]) + (mrg[2 * kTM + lr] + mrg[3 * kTM + lr]);
   cta_teardown(ctl, tbase);
+}
+
+// ---------------------------------------------------------------- pass 2, 256 keys per CTA
+// The held keys are the MMA's B (N = 256), a streamed query block its A: an accumulator lane is a query row, so
+// that a thread's row statistics are two registers (the 128-key kernel reads two of them per column pair from
+// shared memory) and its 64 columns' sums stay in registers over all the query blocks; rows are summed
+// across lanes once, at the end.  Each query block is read for 256 keys.  Bound by the tensor cores, which power
+// holds near 1.5 PFLOP/s, and the exponentials: batch 2, 32/8 heads, D 128, T = 16384 1.53 ms, 1.87 with the
+// 128-key kernel.  Registers: 18 warps of 96 would spill the sums, so four warps (two of them idle) give theirs
+// up: 4 x 32 + 16 x 112 = 20 x 96.
+constexpr int kWideCh = 32;             // accumulator columns read at a time
+constexpr int kWideRegRole = 32, kWideRegEpi = 112;
+constexpr int kWideThr = (4 + kEpiWarps) * 32;   // two role warps, two idle ones, the epilogue's
+template <int D>
+struct WideLayout {
+  static constexpr int kS = 4, kNB = 2, kTN = 256;
+  static constexpr int ATOM_A = kTM * 128, ATOM_B = kTN * 128;
+  static constexpr int TILE_A = (D / 64) * ATOM_A, TILE_B = (D / 64) * ATOM_B;
+  static constexpr int S_OFF = TILE_B;                    // [kS] streamed query blocks
+  static constexpr int ST_OFF = S_OFF + kS * TILE_A;      // [kS] their statistics
+  static constexpr int MRG_OFF = ST_OFF + kS * kStatBytes;   // [4][kTN] lane quarters' sums
+  static constexpr int CTL_OFF = MRG_OFF + 4 * kTN * 4;
+  static constexpr int BYTES = CTL_OFF + 256;
+  static constexpr int ALLOC = BYTES + 1024;
+};
+struct WideCtl {
+  uint64_t full[4], empty[4], sempty[4], tfull[2], tempty[2], abar;
+  uint32_t tslot;
+  int fail, issued, mma_issued;
+};
+
+template <int D>
+__global__ void __launch_bounds__(kWideThr, 1)
+    colsum_wide_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant__ CUtensorMap kmap,
+                       const ScoreArgs a) {
+  using L = WideLayout<D>;
+  constexpr int kS = L::kS, kNB = L::kNB, kTN = L::kTN;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* sm = align1024(smem_raw);
+  WideCtl* ctl = reinterpret_cast<WideCtl*>(sm + L::CTL_OFF);
+  volatile int* fail = &ctl->fail;
+  const int bh = (int)blockIdx.x;                        // the key blocks that the most rows see first
+  const int b = bh / a.Hkv, kvh = bh % a.Hkv;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int lq = warp & 3, cg = (warp - 4) >> 2;         // (epilogue warps) lane quarter, 64-column group
+  const int lr = lq * 32 + lane;                         // accumulator lane = row of the query block
+  const int64_t j0 = (int64_t)blockIdx.y * kTN;
+  const int rb_begin = (int)(std::max<int64_t>(0, j0 - a.pos0) / a.rpb);
+  const int ntiles = std::max(0, a.rowblocks - rb_begin);
+  const float2* stats = a.row_st + (int64_t)bh * a.rowblocks * a.n_ksplit * kTM;
+
+  if (warp == 0) tc_alloc(&ctl->tslot, kNB * kTN);
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < kS; ++i) {
+      tc_mbar_init(&ctl->full[i], 1);
+      tc_mbar_init(&ctl->empty[i], 1);
+      tc_mbar_init(&ctl->sempty[i], kEpiWarps);
+    }
+    for (int i = 0; i < kNB; ++i) {
+      tc_mbar_init(&ctl->tfull[i], 1);
+      tc_mbar_init(&ctl->tempty[i], kEpiWarps);
+    }
+    tc_mbar_init(&ctl->abar, 1);
+    tc_fence_mbar_init();
+    ctl->fail = ctl->issued = ctl->mma_issued = 0;
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tbase = ctl->tslot;
+
+  if (warp < 4) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;\n" ::"n"(kWideRegRole) : "memory");
+    if (warp == 0 && lane == 0) {         // producer
+      tc_mbar_expect_tx(&ctl->abar, L::TILE_B);
+      for (int at = 0; at < D / 64; ++at)
+        tma_load_4d(sm + at * L::ATOM_B, &kmap, at * 64, (int)j0, kvh, b, &ctl->abar);
+      for (int t = 0; t < ntiles; ++t) {
+        const int s = t % kS, n = t / kS;
+        if (n > 0) {
+          if (!role_wait(&ctl->empty[s], (uint32_t)((n - 1) & 1), fail)) break;
+          if (!role_wait(&ctl->sempty[s], (uint32_t)((n - 1) & 1), fail)) break;
+        }
+        const int rb = rb_begin + t;
+        tc_mbar_expect_tx(&ctl->full[s], (uint32_t)(L::TILE_A + kStatBytes));
+        for (int at = 0; at < D / 64; ++at)
+          tma_load_4d(sm + L::S_OFF + s * L::TILE_A + at * L::ATOM_A, &qmap, at * 64, rb * a.rpb, kvh * a.G, b,
+                      &ctl->full[s]);
+        bulk_load(sm + L::ST_OFF + s * kStatBytes, stats + (int64_t)rb * a.n_ksplit * kTM, kStatBytes, &ctl->full[s]);
+        ctl->issued = t + 1;
+      }
+    }
+    if (warp == 1 && lane == 0) {         // MMA issuer
+      const uint64_t held = tc_desc_sw128(smem_addr(sm)), st = tc_desc_sw128(smem_addr(sm + L::S_OFF));
+      if (role_wait(&ctl->abar, 0, fail)) {
+        for (int t = 0; t < ntiles; ++t) {
+          const int s = t % kS, bf = t % kNB, u = t / kNB;
+          if (!role_wait(&ctl->full[s], (uint32_t)((t / kS) & 1), fail)) break;
+          if (u > 0 && !role_wait(&ctl->tempty[bf], (uint32_t)((u - 1) & 1), fail)) break;
+          tc_fence_after();
+          issue_tile<D, kTN>(tbase + (uint32_t)(bf * kTN), st + (uint64_t)((s * L::TILE_A) >> 4), held);
+          tc_commit(&ctl->empty[s]);
+          tc_commit(&ctl->tfull[bf]);
+          ctl->mma_issued = t + 1;
+        }
+      }
+    }
+  } else {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;\n" ::"n"(kWideRegEpi) : "memory");
+    const uint64_t sc2 = pk2(a.scale_log2, a.scale_log2);
+    uint64_t acc[32];                     // columns cg 64 + 2q, + 1: this row's sums over the query blocks
+#pragma unroll
+    for (int q = 0; q < 32; ++q) acc[q] = 0ull;
+    for (int t = 0; t < ntiles; ++t) {
+      const int s = t % kS, bf = t % kNB;
+      bool ok = role_wait(&ctl->tfull[bf], (uint32_t)((t / kNB) & 1), fail);
+      ok = ok && role_wait(&ctl->full[s], (uint32_t)((t / kS) & 1), fail);   // (the statistics' copy)
+      if (!__all_sync(0xffffffffu, ok)) break;
+      tc_fence_after();
+      const float* st = reinterpret_cast<const float*>(sm + L::ST_OFF + s * kStatBytes) + (lr >> 1) * 4 + (lr & 1);
+      const float nm = st[0], w = st[2];
+      const uint64_t nm2 = pk2(nm, nm), w2 = pk2(w, w);
+      const uint32_t col = tbase + (uint32_t)(bf * kTN + cg * 64) + ((uint32_t)(lq * 32) << 16);
+      const int64_t i0 = (int64_t)(rb_begin + t) * a.rpb;
+      // the last of the CTA's keys that this row sees
+      const int lim = (int)std::min<int64_t>(kTN, a.pos0 + i0 + (lr & (a.rpb - 1)) - j0) - cg * 64;
+      const bool whole = a.pos0 + i0 - j0 >= cg * 64 + 63;   // every row sees the warp's keys
+#pragma unroll
+      for (int ch = 0; ch < 64 / kWideCh; ++ch) {
+        float v[kWideCh];
+        tc_ld32(col + (uint32_t)(ch * kWideCh), v);
+        if (ch == 64 / kWideCh - 1) {
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) {
+            tc_mbar_arrive(&ctl->tempty[bf]);
+            tc_mbar_arrive(&ctl->sempty[s]);
+          }
+        }
+        if (whole) {
+#pragma unroll
+          for (int q = 0; q < kWideCh / 2; ++q) {
+            const float2 x = upk2(ffma2(pk2(v[2 * q], v[2 * q + 1]), sc2, nm2));
+            acc[ch * (kWideCh / 2) + q] = ffma2(pk2(ex2_approx(x.x), ex2_approx(x.y)), w2, acc[ch * (kWideCh / 2) + q]);
+          }
+        } else {
+#pragma unroll
+          for (int q = 0; q < kWideCh / 2; ++q) {
+            const int c = ch * kWideCh + 2 * q;
+            const float2 x = upk2(ffma2(pk2(v[2 * q], v[2 * q + 1]), sc2, nm2));
+            const float p0 = c <= lim ? ex2_approx(x.x) : 0.f, p1 = c + 1 <= lim ? ex2_approx(x.y) : 0.f;
+            acc[ch * (kWideCh / 2) + q] = ffma2(pk2(p0, p1), w2, acc[ch * (kWideCh / 2) + q]);
+          }
+        }
+      }
+    }
+    // the warp's 32 rows summed: halves of the columns change lanes until each lane holds one pair
+#pragma unroll
+    for (int h = 16; h >= 1; h >>= 1) {
+      const bool up = lane & h;
+#pragma unroll
+      for (int q = 0; q < h; ++q) {
+        const uint64_t send = up ? acc[q] : acc[q + h], keep = up ? acc[q + h] : acc[q];
+        acc[q] = fadd2(keep, (uint64_t)__shfl_xor_sync(0xffffffffu, (unsigned long long)send, h));
+      }
+    }
+    // lane bits from 16 down chose the upper half: the lane's pair is number `lane`
+    reinterpret_cast<uint64_t*>(sm + L::MRG_OFF)[lq * (kTN / 2) + cg * 32 + lane] = acc[0];
+  }
+  __syncthreads();
+  const float* mrg = reinterpret_cast<const float*>(sm + L::MRG_OFF);
+  if (threadIdx.x < kTN && j0 + threadIdx.x < a.T)
+    a.score[(int64_t)bh * a.T + j0 + threadIdx.x] = (mrg[threadIdx.x] + mrg[kTN + threadIdx.x]) +
+                                                    (mrg[2 * kTN + threadIdx.x] + mrg[3 * kTN + threadIdx.x]);
+  tc_fence_before();
+  if (threadIdx.x == 0 && ctl->fail) {    // copies and products already issued end before the CTA does
+    tc_mbar_wait(&ctl->abar, 0, kWaitNs);
+    for (int t = std::max(0, ctl->issued - kS); t < ctl->issued; ++t)
+      tc_mbar_wait(&ctl->full[t % kS], (uint32_t)((t / kS) & 1), kWaitNs);
+    if (ctl->mma_issued > 0) {
+      const int t = ctl->mma_issued - 1;
+      tc_mbar_wait(&ctl->tfull[t % kNB], (uint32_t)((t / kNB) & 1), kWaitNs);
+    }
+  }
+  __syncthreads();
+  tc_fence_after();
+  if (warp == 0) tc_dealloc(tbase, kNB * kTN);
 }
 
 // ---------------------------------------------------------------- pass 2 over one query block
@@ -541,7 +746,7 @@ __global__ void __launch_bounds__(kThr, 1)
           tma_load_4d(sm + L::B_OFF + s * L::TILE_B + at * L::ATOM_B, &kmap, at * 64, (int)((t_last - t) * kBlk),
                       kvh, b, bar);
       },
-      [&](int t, uint32_t col, int) {
+      [&](int t, uint32_t col, int, auto release) {
         const int64_t jt = (t_last - t) * kBlk;
         const int64_t jrel = jt + lr - a.pos0;   // rows i >= jrel see this key
         const float4* s4 = reinterpret_cast<const float4*>(sm + L::ST_OFF) + hf * 32;
@@ -567,6 +772,7 @@ __global__ void __launch_bounds__(kThr, 1)
             sp2[q & 1] = fadd2(sp2[q & 1], pk2(p0, p1));
           }
         }
+        release();                        // (earlier, the registers do not suffice)
         const float2 s0 = upk2(sp2[0]), s1 = upk2(sp2[1]);
         const float sum = (s0.x + s0.y) + (s1.x + s1.y);
         if (jt + lr < a.T) {
@@ -613,6 +819,18 @@ cudaError_t make_map(CUtensorMap* m, const void* base, int D, int64_t rows, int6
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
+// Whether the wide kernel is launched with the registers that its warps divide among them (a larger
+// share than that would wait for ever)
+template <int D>
+bool wide_registers() {
+  static const bool ok = [] {
+    cudaFuncAttributes at;
+    return cudaFuncGetAttributes(&at, colsum_wide_kernel<D>) == cudaSuccess &&
+           (at.numRegs + 7) / 8 * 8 * (kWideThr / 32) >= 4 * kWideRegRole + kEpiWarps * kWideRegEpi;
+  }();
+  return ok;
+}
+
 template <int D>
 cudaError_t launch_scores_t(const CUtensorMap& qm, const CUtensorMap& k256, const CUtensorMap& k128,
                             const ScoreArgs& a, int units, int keyblocks, cudaStream_t st) {
@@ -620,11 +838,19 @@ cudaError_t launch_scores_t(const CUtensorMap& qm, const CUtensorMap& k256, cons
   constexpr int smem1 = std::max(Layout<D, kTN1>::ALLOC, 116 * 1024);
   constexpr int smem2 = std::max(Layout<D, kTN2>::ALLOC, 116 * 1024);
   static_assert(smem1 <= 227 * 1024 && smem2 <= 227 * 1024, "shared memory");
-  cudaError_t e = cudaFuncSetAttribute(rowstats_tc_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem1);
+  constexpr int smem1w = std::max(Layout<D, kTN1, 2>::ALLOC, 116 * 1024);
+  cudaError_t e = cudaFuncSetAttribute(rowstats_tc_kernel<D, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem1);
+  if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(rowstats_tc_kernel<D, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem1w);
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(colsum_tc_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem2);
   if (e != cudaSuccess) return e;
-  rowstats_tc_kernel<D><<<dim3(a.n_ksplit, a.rowblocks, units), kThr, smem1, st>>>(qm, k256, a);
+  // Two row blocks per CTA from 1.5 waves of pairs: 256 pairs (16/2 heads, T = 4096) 194 -> 188 us, 188 pairs
+  // (T = 3000) 151 -> 155; below, the longest CTA is the time.
+  if (a.n_ksplit == 1 && (int64_t)units * ceil_div(a.rowblocks, 2) * 2 >= 3 * kNumSMs && a.rowblocks > 1)
+    rowstats_tc_kernel<D, 2><<<dim3(units, (unsigned)ceil_div(a.rowblocks, 2)), kThr, smem1w, st>>>(qm, k256, a);
+  else
+    rowstats_tc_kernel<D, 1><<<dim3(a.n_ksplit, a.rowblocks, units), kThr, smem1, st>>>(qm, k256, a);
   e = cudaPeekAtLastError();
   if (e != cudaSuccess) return e;
   if (a.rowblocks == 1) {                 // one query block: hold it, stream pass 1's key splits
@@ -638,6 +864,17 @@ cudaError_t launch_scores_t(const CUtensorMap& qm, const CUtensorMap& k256, cons
                                                                             a.rowblocks, a.R);
   e = cudaPeekAtLastError();
   if (e != cudaSuccess) return e;
+  // 256 keys per CTA when these make more than one wave: 256 CTAs (32/8 heads, batch 4, T = 2048) 204 -> 174 us,
+  // 128 (batch 1, T = 4096) 191 -> 202.
+  const int64_t wide = ceil_div(a.T, WideLayout<D>::kTN);
+  if (units * wide > kNumSMs && wide <= 65535 && wide_registers<D>()) {
+    constexpr int smem3 = std::max(WideLayout<D>::ALLOC, 116 * 1024);
+    static_assert(smem3 <= 227 * 1024, "shared memory");
+    e = cudaFuncSetAttribute(colsum_wide_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem3);
+    if (e != cudaSuccess) return e;
+    colsum_wide_kernel<D><<<dim3(units, (unsigned)wide), kWideThr, smem3, st>>>(qm, k256, a);
+    return cudaPeekAtLastError();
+  }
   colsum_tc_kernel<D><<<dim3(keyblocks, units), kThr, smem2, st>>>(qm, k128, a);
   return cudaPeekAtLastError();
 }
