@@ -27,9 +27,9 @@
 //   warps 2..17 read finished accumulators in two groups of eight: group g takes the products
 //           t = g mod 2, so the groups work a product apart and one group's exponentials overlap the
 //           other's loads and reductions; warp w reads lanes 32 (w % 4) .. + 31 (the lane quarter it
-//           may access) and one half of the product's columns, 64 at a time (the 256-key kernel: all
-//           sixteen take every product, a quarter of its columns each).  A buffer is given back as soon as
-//           it is read, before the exponentials of what was read.
+//           may access) and one half of the product's columns, 64 at a time.  With two held row blocks or
+//           256 held keys all sixteen take every product, a quarter of its 256 columns each.  A buffer is
+//           given back as soon as it is read, before the exponentials of what was read.
 // Loads, products and epilogues of different tiles overlap; nothing in the tile loop waits on a
 // CTA-wide barrier.  Every wait is bounded (1 s of the GPU's global timer): on a timeout the role
 // raises MKV_FLAG_WAIT_TIMEOUT and sets a flag that ends the other roles' waits; the CTA then waits
@@ -159,7 +159,7 @@ __device__ __forceinline__ void issue_tile(uint32_t d_tmem, uint64_t a, uint64_t
 
 // Barriers and tensor memory of a CTA; returns the tensor-memory base (all 512 columns).
 template <int TN>
-__device__ __forceinline__ uint32_t cta_setup(Ctl<TN>* ctl) {
+__device__ __forceinline__ uint32_t cta_setup(Ctl<TN>* ctl, int readers = kGroupWarps) {
   using C = Tiling<TN>;
   if ((threadIdx.x >> 5) == 0) tc_alloc(&ctl->tslot, C::kNB * TN);
   if (threadIdx.x == 0) {
@@ -170,7 +170,7 @@ __device__ __forceinline__ uint32_t cta_setup(Ctl<TN>* ctl) {
     }
     for (int b = 0; b < C::kNB; ++b) {
       tc_mbar_init(&ctl->tfull[b], 1);
-      tc_mbar_init(&ctl->tempty[b], kGroupWarps);
+      tc_mbar_init(&ctl->tempty[b], readers);
     }
     tc_mbar_init(&ctl->abar, 1);
     tc_fence_mbar_init();
@@ -205,9 +205,9 @@ __device__ __forceinline__ void cta_teardown(Ctl<TN>* ctl, uint32_t tbase) {
 }
 
 // The three roles over `ntiles` streamed tiles.  issue_a(bar) loads the held operand, or both (kHeld = 2:
-// each tile then gives two products, the second held operand's after the first's, one per epilogue
-// group); issue_b(t, s, bar) loads tile t into stage s; epi(t, col, s, release) reads the thread's half of a
-// product (kHalf columns from tensor-memory address col, lane 0), calls release() once that is read and,
+// each tile then gives two products, and all sixteen epilogue warps read a quarter of each: epi's last
+// argument but one is then the held operand); issue_b(t, s, bar) loads tile t into stage s; epi(t, col, s, release) reads the thread's half of a
+// product (kHalf columns, or the quarter, from tensor-memory address col, lane 0), calls release() once that is read and,
 // with kStats, uses the statistics of stage s.  With kStreamA the streamed tile is the MMA's A operand and
 // the held one its B (the accumulator's lanes then follow the streamed rows).
 template <int D, int TN, bool kStats, bool kStreamA = false, int kHeld = 1, typename IssueA, typename IssueB, typename Epi>
@@ -264,9 +264,27 @@ __device__ __forceinline__ void run_roles(uint8_t* sm, Ctl<TN>* ctl, uint32_t tb
     // the held operand's phase: what came with it (statistics held beside it) is visible after it
     const bool held = role_wait(&ctl->abar, 0, fail);
     if (!__all_sync(0xffffffffu, held)) return;
-    for (int x = grp; x < kHeld * ntiles; x += 2) {   // (two held operands: one per group)
-      const int t = x / kHeld, s = t % kS, bf = x % kNB;
-      bool ok = role_wait(&ctl->tfull[bf], (uint32_t)((x / kNB) & 1), fail);
+    if constexpr (kHeld == 2) {           // every warp takes a quarter of every product's columns
+      const int quarter = (warp - 2) >> 2;
+      for (int t = 0; t < ntiles; ++t) {
+        bool ok = true;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          ok = role_wait(&ctl->tfull[h], (uint32_t)(t & 1), fail);
+          ok = __all_sync(0xffffffffu, ok);
+          if (!ok) break;
+          tc_fence_after();
+          epi(t, tbase + (uint32_t)(h * TN + quarter * (TN / 4)), h, [&]() {
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) tc_mbar_arrive(&ctl->tempty[h]);
+          });
+        }
+        if (!ok) break;
+      }
+    } else for (int t = grp; t < ntiles; t += 2) {
+      const int s = t % kS, bf = t % kNB;
+      bool ok = role_wait(&ctl->tfull[bf], (uint32_t)((t / kNB) & 1), fail);
       // the statistics came with the stage's operand: their copy completed that phase of full[s]
       if (kStats) ok = ok && role_wait(&ctl->full[s], (uint32_t)((t / kS) & 1), fail);
       if (!__all_sync(0xffffffffu, ok)) break;
@@ -285,10 +303,12 @@ __device__ __forceinline__ void run_roles(uint8_t* sm, Ctl<TN>* ctl, uint32_t tb
 }
 
 // ---------------------------------------------------------------- pass 1
-// HELD = 2: two row blocks per CTA, a key tile read once for both.  Bound by L2 reads and the products' waits
-// before the exponentials: 32/8 heads, D 128, batch 16, T = 512 (1024 block pairs): both passes 132.9 us with
-// one block per CTA, 112.3 with two; batch 4, T = 2048: 228 and 204.  (Giving the buffers back early: batch 2,
-// T = 16384 3.85 -> 3.65 ms.)
+// HELD = 2: two row blocks per CTA, a key tile read once for both, and each product's buffer given back after
+// one read of 64 columns a thread (one block: after the exponentials of the first 64 of 128).  Bound by the
+// tensor cores under the power limit and the wait for each product.  Both passes, 32/8 heads, D 128:
+// batch 16, T = 512 (1024 block pairs) 132.9 us with one block per CTA, 112.3 with two; batch 2, T = 16384
+// 3.20 ms with half the warps per product (a group to each block), 3.06 with all.  (Giving the buffers back
+// early at all: 3.85 -> 3.65 ms.)
 template <int D, int HELD>
 __global__ void __launch_bounds__(kThr, 1)
     rowstats_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant__ CUtensorMap kmap,
@@ -307,18 +327,23 @@ __global__ void __launch_bounds__(kThr, 1)
   const int hf = cq & 1;                                 // column half of the tile
   const int lr = lq * 32 + (threadIdx.x & 31);           // accumulator lane = query row of the block
 
-  const int rb = rb0 + (HELD == 2 ? cq >> 1 : 0);        // (epilogue warps) the group's row block
   // the last valid row bounds the causal key range
   const int64_t row_hi = std::min<int64_t>((int64_t)(rb0 + HELD) * a.rpb, a.R);   // exclusive
   const int64_t k_begin = (int64_t)ks * a.tiles_per_split * kTN;
   const int64_t k_end = std::min<int64_t>(std::min<int64_t>(k_begin + (int64_t)a.tiles_per_split * kTN, a.T),
                                           a.pos0 + row_hi);
   const int ntiles = k_end > k_begin ? (int)ceil_div_dev(k_end - k_begin, kTN) : 0;
-  const int64_t irow = (int64_t)rb * a.rpb + (lr & (a.rpb - 1));
-  const int64_t lim = irow < a.R ? std::min<int64_t>(k_end - 1, a.pos0 + irow) : -1;   // last key it sees
+  int64_t lim[HELD];                      // the last key that the thread's row (of each block) sees
+#pragma unroll
+  for (int h = 0; h < HELD; ++h) {
+    const int64_t irow = (int64_t)(rb0 + h) * a.rpb + (lr & (a.rpb - 1));
+    lim[h] = irow < a.R ? std::min<int64_t>(k_end - 1, a.pos0 + irow) : -1;
+  }
 
-  const uint32_t tbase = cta_setup(ctl);
-  float m_run = -INFINITY, l_run = 0.f;
+  const uint32_t tbase = cta_setup(ctl, HELD == 2 ? kEpiWarps : kGroupWarps);
+  float m_run[HELD], l_run[HELD];
+#pragma unroll
+  for (int h = 0; h < HELD; ++h) m_run[h] = -INFINITY, l_run[h] = 0.f;
   run_roles<D, kTN1, false, false, HELD>(
       sm, ctl, tbase, ntiles,
       [&](uint64_t* bar) {                // one box of G heads x rpb rows: head g's rows are tile rows g rpb ..
@@ -333,22 +358,25 @@ __global__ void __launch_bounds__(kThr, 1)
           tma_load_4d(sm + L::B_OFF + s * L::TILE_B + at * L::ATOM_B, &kmap, at * 64,
                       (int)(k_begin + (int64_t)t * kTN), kvh, b, bar);
       },
-      [&](int t, uint32_t col, int, auto release) {
+      [&](int t, uint32_t col, int hs, auto release) {
+        const int h = HELD == 2 ? hs : 0;   // the held block; its warp's columns of the tile
+        constexpr int kCols = HELD == 2 ? kTN / 4 : kHalf;
+        const int c0 = HELD == 2 ? cq * kCols : hf * kHalf;
 #pragma unroll 1
-        for (int ch = 0; ch < kHalf / 64; ++ch) {
-          const int64_t jc = k_begin + (int64_t)t * kTN + hf * kHalf + ch * 64;
+        for (int ch = 0; ch < kCols / 64; ++ch) {
+          const int64_t jc = k_begin + (int64_t)t * kTN + c0 + ch * 64;
           float v[64];
           tc_ld64(col + ((uint32_t)(lq * 32) << 16) + (uint32_t)(ch * 64), v);
-          if (ch == kHalf / 64 - 1) release();
-          if (jc + 63 > lim) {            // keys past the row's causal limit (or the range) drop out
+          if (ch == kCols / 64 - 1) release();
+          if (jc + 63 > lim[h]) {            // keys past the row's causal limit (or the range) drop out
 #pragma unroll
-            for (int e = 0; e < 64; ++e) v[e] = jc + e <= lim ? v[e] : -INFINITY;
+            for (int e = 0; e < 64; ++e) v[e] = jc + e <= lim[h] ? v[e] : -INFINITY;
           }
           float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};   // max of the raw products
 #pragma unroll
           for (int q = 0; q < 32; ++q) mx[q & 3] = fmax3(mx[q & 3], v[2 * q], v[2 * q + 1]);
           // the scale is positive: the max of the scaled products is the scaled max
-          const float m_new = fmaxf(m_run, fmax3(mx[0], mx[1], fmaxf(mx[2], mx[3])) * a.scale_log2);
+          const float m_new = fmaxf(m_run[h], fmax3(mx[0], mx[1], fmaxf(mx[2], mx[3])) * a.scale_log2);
           if (m_new != -INFINITY) {
             // 2^(s scale - m) and its sum, two columns per packed instruction
             const uint64_t sc2 = pk2(a.scale_log2, a.scale_log2), nm2 = pk2(-m_new, -m_new);
@@ -359,29 +387,32 @@ __global__ void __launch_bounds__(kThr, 1)
               sp2[q & 1] = fadd2(sp2[q & 1], pk2(ex2_approx(x.x), ex2_approx(x.y)));
             }
             const float2 s0 = upk2(sp2[0]), s1 = upk2(sp2[1]);
-            l_run = l_run * ex2_approx(m_run - m_new) + ((s0.x + s0.y) + (s1.x + s1.y));
-            m_run = m_new;
+            l_run[h] = l_run[h] * ex2_approx(m_run[h] - m_new) + ((s0.x + s0.y) + (s1.x + s1.y));
+            m_run[h] = m_new;
           }
         }
       });
-  // the partials of each row (from the column halves; one held operand: and the groups) merged into this split's (m, l)
+  // the four partials of each row (groups and column halves, or column quarters) merged into this split's (m, l)
   float2* mrg = reinterpret_cast<float2*>(sm + L::MRG_OFF);
-  if (warp >= 2) mrg[cq * kTM + lr] = make_float2(m_run, l_run);
-  __syncthreads();
-  constexpr int NP = 4 / HELD;
-  if (warp >= 2 && cq % NP == 0 && rb < a.rowblocks) {
-    float M = -INFINITY;
 #pragma unroll
-    for (int q = 0; q < NP; ++q) M = fmaxf(M, mrg[(cq + q) * kTM + lr].x);
-    float l = 0.f;
-    if (M != -INFINITY) {
+  for (int h = 0; h < HELD; ++h) {
+    if (h > 0) __syncthreads();
+    if (warp >= 2) mrg[cq * kTM + lr] = make_float2(m_run[h], l_run[h]);
+    __syncthreads();
+    if (warp >= 2 && cq == 0 && rb0 + h < a.rowblocks) {
+      float M = -INFINITY;
 #pragma unroll
-      for (int q = 0; q < NP; ++q) {
-        const float2 o = mrg[(cq + q) * kTM + lr];
-        l += o.y * ex2_approx(o.x - M);
+      for (int q = 0; q < 4; ++q) M = fmaxf(M, mrg[q * kTM + lr].x);
+      float l = 0.f;
+      if (M != -INFINITY) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const float2 o = mrg[q * kTM + lr];
+          l += o.y * ex2_approx(o.x - M);
+        }
       }
+      a.row_st[(((int64_t)bh * a.rowblocks + rb0 + h) * a.n_ksplit + ks) * kTM + lr] = make_float2(M, l);
     }
-    a.row_st[(((int64_t)bh * a.rowblocks + rb) * a.n_ksplit + ks) * kTM + lr] = make_float2(M, l);
   }
   cta_teardown(ctl, tbase);
 }
