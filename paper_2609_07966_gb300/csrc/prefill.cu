@@ -27,9 +27,9 @@
 //   warps 2..17 read finished accumulators in two groups of eight: group g takes the products
 //           t = g mod 2, so the groups work a product apart and one group's exponentials overlap the
 //           other's loads and reductions; warp w reads lanes 32 (w % 4) .. + 31 (the lane quarter it
-//           may access) and one half of the product's columns, 64 at a time.  With two held row blocks or
-//           256 held keys all sixteen take every product, a quarter of its 256 columns each.  A buffer is
-//           given back as soon as it is read, before the exponentials of what was read.
+//           may access) and one half of the product's columns, 64 at a time.  Products of 256 columns are
+//           taken by all sixteen, a quarter of the columns each.  A buffer is given back as soon as it is
+//           read, before the exponentials of what was read.
 // Loads, products and epilogues of different tiles overlap; nothing in the tile loop waits on a
 // CTA-wide barrier.  Every wait is bounded (1 s of the GPU's global timer): on a timeout the role
 // raises MKV_FLAG_WAIT_TIMEOUT and sets a flag that ends the other roles' waits; the CTA then waits
@@ -74,7 +74,8 @@ struct Tiling {
   static constexpr int kTN = TN;
   static constexpr int kNB = 512 / TN;            // accumulator buffers: all 512 tensor-memory columns
   static constexpr int kS = TN == 256 ? 2 : 4;    // operand stages
-  static constexpr int kHalf = TN / 2;            // accumulator columns an epilogue warp reads per tile
+  static constexpr bool kAll = TN == 256;         // all epilogue warps read each product (else: a group of them)
+  static constexpr int kCols = kAll ? TN / 4 : TN / 2;   // accumulator columns an epilogue warp reads of it
   static constexpr int kBlocks = TN / kBlk;       // query blocks per tile (pass 2)
 };
 constexpr int kTN1 = 256;                // pass 1's tile
@@ -159,7 +160,7 @@ __device__ __forceinline__ void issue_tile(uint32_t d_tmem, uint64_t a, uint64_t
 
 // Barriers and tensor memory of a CTA; returns the tensor-memory base (all 512 columns).
 template <int TN>
-__device__ __forceinline__ uint32_t cta_setup(Ctl<TN>* ctl, int readers = kGroupWarps) {
+__device__ __forceinline__ uint32_t cta_setup(Ctl<TN>* ctl) {
   using C = Tiling<TN>;
   if ((threadIdx.x >> 5) == 0) tc_alloc(&ctl->tslot, C::kNB * TN);
   if (threadIdx.x == 0) {
@@ -170,7 +171,7 @@ __device__ __forceinline__ uint32_t cta_setup(Ctl<TN>* ctl, int readers = kGroup
     }
     for (int b = 0; b < C::kNB; ++b) {
       tc_mbar_init(&ctl->tfull[b], 1);
-      tc_mbar_init(&ctl->tempty[b], readers);
+      tc_mbar_init(&ctl->tempty[b], C::kAll ? kEpiWarps : kGroupWarps);
     }
     tc_mbar_init(&ctl->abar, 1);
     tc_fence_mbar_init();
@@ -205,17 +206,16 @@ __device__ __forceinline__ void cta_teardown(Ctl<TN>* ctl, uint32_t tbase) {
 }
 
 // The three roles over `ntiles` streamed tiles.  issue_a(bar) loads the held operand, or both (kHeld = 2:
-// each tile then gives two products, and all sixteen epilogue warps read a quarter of each: epi's last
-// argument but one is then the held operand); issue_b(t, s, bar) loads tile t into stage s; epi(t, col, s, release) reads the thread's half of a
-// product (kHalf columns, or the quarter, from tensor-memory address col, lane 0), calls release() once that is read and,
-// with kStats, uses the statistics of stage s.  With kStreamA the streamed tile is the MMA's A operand and
+// each tile then gives two products; epi's third argument is then the held operand); issue_b(t, s, bar) loads tile t into stage s; epi(t, col, s, release) reads the thread's kCols
+// columns of a product (from tensor-memory address col, lane 0), calls release() once that is read and, with
+// kStats, uses the statistics of stage s.  With kStreamA the streamed tile is the MMA's A operand and
 // the held one its B (the accumulator's lanes then follow the streamed rows).
 template <int D, int TN, bool kStats, bool kStreamA = false, int kHeld = 1, typename IssueA, typename IssueB, typename Epi>
 __device__ __forceinline__ void run_roles(uint8_t* sm, Ctl<TN>* ctl, uint32_t tbase, int ntiles, IssueA issue_a,
                                           IssueB issue_b, Epi epi) {
   using L = Layout<D, TN, kHeld>;
   using C = Tiling<TN>;
-  constexpr int kS = C::kS, kNB = C::kNB, kHalf = C::kHalf;
+  constexpr int kS = C::kS, kNB = C::kNB;
   volatile int* fail = &ctl->fail;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (ntiles <= 0) return;
@@ -264,20 +264,21 @@ __device__ __forceinline__ void run_roles(uint8_t* sm, Ctl<TN>* ctl, uint32_t tb
     // the held operand's phase: what came with it (statistics held beside it) is visible after it
     const bool held = role_wait(&ctl->abar, 0, fail);
     if (!__all_sync(0xffffffffu, held)) return;
-    if constexpr (kHeld == 2) {           // every warp takes a quarter of every product's columns
+    if constexpr (C::kAll) {              // every warp takes a quarter of every product's columns
       const int quarter = (warp - 2) >> 2;
       for (int t = 0; t < ntiles; ++t) {
         bool ok = true;
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          ok = role_wait(&ctl->tfull[h], (uint32_t)(t & 1), fail);
+        for (int h = 0; h < kHeld; ++h) {
+          const int x = t * kHeld + h, bf = x % kNB;
+          ok = role_wait(&ctl->tfull[bf], (uint32_t)((x / kNB) & 1), fail);
           ok = __all_sync(0xffffffffu, ok);
           if (!ok) break;
           tc_fence_after();
-          epi(t, tbase + (uint32_t)(h * TN + quarter * (TN / 4)), h, [&]() {
+          epi(t, tbase + (uint32_t)(bf * TN + quarter * (TN / 4)), h, [&]() {
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) tc_mbar_arrive(&ctl->tempty[h]);
+            if (lane == 0) tc_mbar_arrive(&ctl->tempty[bf]);
           });
         }
         if (!ok) break;
@@ -289,7 +290,7 @@ __device__ __forceinline__ void run_roles(uint8_t* sm, Ctl<TN>* ctl, uint32_t tb
       if (kStats) ok = ok && role_wait(&ctl->full[s], (uint32_t)((t / kS) & 1), fail);
       if (!__all_sync(0xffffffffu, ok)) break;
       tc_fence_after();
-      epi(t, tbase + (uint32_t)(bf * TN + half * kHalf), s, [&]() {
+      epi(t, tbase + (uint32_t)(bf * TN + half * C::kCols), s, [&]() {
         tc_fence_before();
         __syncwarp();
         if (lane == 0) tc_mbar_arrive(&ctl->tempty[bf]);
@@ -313,7 +314,8 @@ template <int D, int HELD>
 __global__ void __launch_bounds__(kThr, 1)
     rowstats_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant__ CUtensorMap kmap,
                        const ScoreArgs a) {
-  constexpr int kTN = kTN1, kHalf = Tiling<kTN1>::kHalf;
+  constexpr int kTN = kTN1;
+  static_assert(Tiling<kTN1>::kCols == 64, "one read of 64 columns");
   using L = Layout<D, kTN1, HELD>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* sm = align1024(smem_raw);
@@ -323,8 +325,7 @@ __global__ void __launch_bounds__(kThr, 1)
   const int bh = HELD == 2 ? (int)blockIdx.x : (int)blockIdx.z;
   const int b = bh / a.Hkv, kvh = bh % a.Hkv;
   const int warp = threadIdx.x >> 5;
-  const int lq = warp & 3, cq = (warp - 2) >> 2;         // (epilogue warps) lane quarter; group x half
-  const int hf = cq & 1;                                 // column half of the tile
+  const int lq = warp & 3, cq = (warp - 2) >> 2;         // (epilogue warps) lane quarter; column quarter
   const int lr = lq * 32 + (threadIdx.x & 31);           // accumulator lane = query row of the block
 
   // the last valid row bounds the causal key range
@@ -340,7 +341,7 @@ __global__ void __launch_bounds__(kThr, 1)
     lim[h] = irow < a.R ? std::min<int64_t>(k_end - 1, a.pos0 + irow) : -1;
   }
 
-  const uint32_t tbase = cta_setup(ctl, HELD == 2 ? kEpiWarps : kGroupWarps);
+  const uint32_t tbase = cta_setup(ctl);
   float m_run[HELD], l_run[HELD];
 #pragma unroll
   for (int h = 0; h < HELD; ++h) m_run[h] = -INFINITY, l_run[h] = 0.f;
@@ -358,41 +359,35 @@ __global__ void __launch_bounds__(kThr, 1)
           tma_load_4d(sm + L::B_OFF + s * L::TILE_B + at * L::ATOM_B, &kmap, at * 64,
                       (int)(k_begin + (int64_t)t * kTN), kvh, b, bar);
       },
-      [&](int t, uint32_t col, int hs, auto release) {
-        const int h = HELD == 2 ? hs : 0;   // the held block; its warp's columns of the tile
-        constexpr int kCols = HELD == 2 ? kTN / 4 : kHalf;
-        const int c0 = HELD == 2 ? cq * kCols : hf * kHalf;
-#pragma unroll 1
-        for (int ch = 0; ch < kCols / 64; ++ch) {
-          const int64_t jc = k_begin + (int64_t)t * kTN + c0 + ch * 64;
-          float v[64];
-          tc_ld64(col + ((uint32_t)(lq * 32) << 16) + (uint32_t)(ch * 64), v);
-          if (ch == kCols / 64 - 1) release();
-          if (jc + 63 > lim[h]) {            // keys past the row's causal limit (or the range) drop out
+      [&](int t, uint32_t col, int h, auto release) {   // h: the held block
+        const int64_t jc = k_begin + (int64_t)t * kTN + cq * 64;
+        float v[64];
+        tc_ld64(col + ((uint32_t)(lq * 32) << 16), v);
+        release();
+        if (jc + 63 > lim[h]) {            // keys past the row's causal limit (or the range) drop out
 #pragma unroll
-            for (int e = 0; e < 64; ++e) v[e] = jc + e <= lim[h] ? v[e] : -INFINITY;
+          for (int e = 0; e < 64; ++e) v[e] = jc + e <= lim[h] ? v[e] : -INFINITY;
+        }
+        float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};   // max of the raw products
+#pragma unroll
+        for (int q = 0; q < 32; ++q) mx[q & 3] = fmax3(mx[q & 3], v[2 * q], v[2 * q + 1]);
+        // the scale is positive: the max of the scaled products is the scaled max
+        const float m_new = fmaxf(m_run[h], fmax3(mx[0], mx[1], fmaxf(mx[2], mx[3])) * a.scale_log2);
+        if (m_new != -INFINITY) {
+          // 2^(s scale - m) and its sum, two columns per packed instruction
+          const uint64_t sc2 = pk2(a.scale_log2, a.scale_log2), nm2 = pk2(-m_new, -m_new);
+          uint64_t sp2[2] = {0ull, 0ull};
+#pragma unroll
+          for (int q = 0; q < 32; ++q) {
+            const float2 x = upk2(ffma2(pk2(v[2 * q], v[2 * q + 1]), sc2, nm2));
+            sp2[q & 1] = fadd2(sp2[q & 1], pk2(ex2_approx(x.x), ex2_approx(x.y)));
           }
-          float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};   // max of the raw products
-#pragma unroll
-          for (int q = 0; q < 32; ++q) mx[q & 3] = fmax3(mx[q & 3], v[2 * q], v[2 * q + 1]);
-          // the scale is positive: the max of the scaled products is the scaled max
-          const float m_new = fmaxf(m_run[h], fmax3(mx[0], mx[1], fmaxf(mx[2], mx[3])) * a.scale_log2);
-          if (m_new != -INFINITY) {
-            // 2^(s scale - m) and its sum, two columns per packed instruction
-            const uint64_t sc2 = pk2(a.scale_log2, a.scale_log2), nm2 = pk2(-m_new, -m_new);
-            uint64_t sp2[2] = {0ull, 0ull};
-#pragma unroll
-            for (int q = 0; q < 32; ++q) {
-              const float2 x = upk2(ffma2(pk2(v[2 * q], v[2 * q + 1]), sc2, nm2));
-              sp2[q & 1] = fadd2(sp2[q & 1], pk2(ex2_approx(x.x), ex2_approx(x.y)));
-            }
-            const float2 s0 = upk2(sp2[0]), s1 = upk2(sp2[1]);
-            l_run[h] = l_run[h] * ex2_approx(m_run[h] - m_new) + ((s0.x + s0.y) + (s1.x + s1.y));
-            m_run[h] = m_new;
-          }
+          const float2 s0 = upk2(sp2[0]), s1 = upk2(sp2[1]);
+          l_run[h] = l_run[h] * ex2_approx(m_run[h] - m_new) + ((s0.x + s0.y) + (s1.x + s1.y));
+          m_run[h] = m_new;
         }
       });
-  // the four partials of each row (groups and column halves, or column quarters) merged into this split's (m, l)
+  // the four partials of each row (column quarters) merged into this split's (m, l)
   float2* mrg = reinterpret_cast<float2*>(sm + L::MRG_OFF);
 #pragma unroll
   for (int h = 0; h < HELD; ++h) {
@@ -490,8 +485,8 @@ __global__ void __launch_bounds__(kThr, 1)
         const uint64_t sc2 = pk2(a.scale_log2, a.scale_log2);
         uint64_t sp2[2] = {0ull, 0ull};
 #pragma unroll 1
-        for (int ch = 0; ch < C::kHalf / 64; ++ch) {
-          const int c0 = hf * C::kHalf + ch * 64;   // the chunk's first column of the tile
+        for (int ch = 0; ch < C::kCols / 64; ++ch) {
+          const int c0 = hf * C::kCols + ch * 64;   // the chunk's first column of the tile
           const int h = c0 / kBlk, cin = c0 % kBlk;   // its query block and first column in the block
           const int rb = rb_begin + C::kBlocks * t + h;
           const int64_t i0 = (int64_t)rb * a.rpb;   // row index of the block's first row per head
@@ -514,9 +509,9 @@ __global__ void __launch_bounds__(kThr, 1)
               const float4 w = s4[q];
               const int c = cin + 2 * q;
               const float2 x = upk2(ffma2(pk2(v[2 * q], v[2 * q + 1]), sc2, pk2(w.x, w.y)));
-              const float p0 = i0 + (c & (a.rpb - 1)) >= jrel ? ex2_approx(x.x) * w.z : 0.f;
-              const float p1 = i0 + ((c + 1) & (a.rpb - 1)) >= jrel ? ex2_approx(x.y) * w.w : 0.f;
-              sp2[q & 1] = fadd2(sp2[q & 1], pk2(p0, p1));
+              const float p0 = i0 + (c & (a.rpb - 1)) >= jrel ? ex2_approx(x.x) : 0.f;
+              const float p1 = i0 + ((c + 1) & (a.rpb - 1)) >= jrel ? ex2_approx(x.y) : 0.f;
+              sp2[q & 1] = ffma2(pk2(p0, p1), pk2(w.z, w.w), sp2[q & 1]);
             }
           }
         }
@@ -798,9 +793,9 @@ __global__ void __launch_bounds__(kThr, 1)
             const float4 w = s4[q];
             const int c = hf * 64 + 2 * q;
             const float2 x = upk2(ffma2(pk2(v[2 * q], v[2 * q + 1]), sc2, pk2(w.x, w.y)));
-            const float p0 = (c & (a.rpb - 1)) >= jrel ? ex2_approx(x.x) * w.z : 0.f;
-            const float p1 = ((c + 1) & (a.rpb - 1)) >= jrel ? ex2_approx(x.y) * w.w : 0.f;
-            sp2[q & 1] = fadd2(sp2[q & 1], pk2(p0, p1));
+            const float p0 = (c & (a.rpb - 1)) >= jrel ? ex2_approx(x.x) : 0.f;
+            const float p1 = ((c + 1) & (a.rpb - 1)) >= jrel ? ex2_approx(x.y) : 0.f;
+            sp2[q & 1] = ffma2(pk2(p0, p1), pk2(w.z, w.w), sp2[q & 1]);
           }
         }
         release();                        // (earlier, the registers do not suffice)
