@@ -206,10 +206,11 @@ __device__ __forceinline__ void cta_teardown(Ctl<TN>* ctl, uint32_t tbase) {
 }
 
 // The three roles over `ntiles` streamed tiles.  issue_a(bar) loads the held operand, or both (kHeld = 2:
-// each tile then gives two products; epi's third argument is then the held operand); issue_b(t, s, bar) loads tile t into stage s; epi(t, col, s, release) reads the thread's kCols
-// columns of a product (from tensor-memory address col, lane 0), calls release() once that is read and, with
-// kStats, uses the statistics of stage s.  With kStreamA the streamed tile is the MMA's A operand and
-// the held one its B (the accumulator's lanes then follow the streamed rows).
+// each tile then gives two products; epi's third argument is then the held operand); issue_b(t, s, bar)
+// loads tile t into stage s; epi(t, col, s, release) reads the thread's kCols columns of a product (from
+// tensor-memory address col, lane 0), calls release() once that is read and, with kStats, uses the
+// statistics of stage s.  With kStreamA the streamed tile is the MMA's A operand and the held one its B (the
+// accumulator's lanes then follow the streamed rows).
 template <int D, int TN, bool kStats, bool kStreamA = false, int kHeld = 1, typename IssueA, typename IssueB, typename Epi>
 __device__ __forceinline__ void run_roles(uint8_t* sm, Ctl<TN>* ctl, uint32_t tbase, int ntiles, IssueA issue_a,
                                           IssueB issue_b, Epi epi) {
