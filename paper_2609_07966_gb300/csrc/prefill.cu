@@ -83,7 +83,8 @@ constexpr int kTN2 = 128;                // pass 2's tile
 
 struct ScoreArgs {
   int64_t R, T, pos0;   // query rows, keys, position of query row 0
-  int Hq, Hkv, G, rpb;  // rpb = rows per head in a 128-row query block (128 / G, a power of two)
+  int Hq, Hkv, G, units;
+  int rpb;              // rpb = rows per head in a 128-row query block (128 / G, a power of two)
   int rowblocks;        // ceil(R / rpb)
   int n_ksplit, tiles_per_split;   // pass 1: key splits and 256-key tiles per split
   float scale_log2;
@@ -323,7 +324,8 @@ __global__ void __launch_bounds__(kThr, 1)
   Ctl<kTN1>* ctl = reinterpret_cast<Ctl<kTN1>*>(sm + L::CTL_OFF);
   const int ks = HELD == 2 ? 0 : blockIdx.x;
   const int rb0 = (a.rowblocks - 1) / HELD * HELD - HELD * (int)blockIdx.y;   // the blocks with the most keys first
-  const int bh = HELD == 2 ? (int)blockIdx.x : (int)blockIdx.z;
+  const int bh = HELD == 2 ? (int)(blockIdx.z * gridDim.x + blockIdx.x) : (int)blockIdx.z;
+  if (HELD == 2 && bh >= a.units) return;
   const int b = bh / a.Hkv, kvh = bh % a.Hkv;
   const int warp = threadIdx.x >> 5;
   const int lq = warp & 3, cq = (warp - 2) >> 2;         // (epilogue warps) lane quarter; column quarter
@@ -567,7 +569,8 @@ __global__ void __launch_bounds__(kWideThr, 1)
   uint8_t* sm = align1024(smem_raw);
   WideCtl* ctl = reinterpret_cast<WideCtl*>(sm + L::CTL_OFF);
   volatile int* fail = &ctl->fail;
-  const int bh = (int)blockIdx.x;                        // the key blocks that the most rows see first
+  const int bh = (int)(blockIdx.z * gridDim.x + blockIdx.x);   // (groups of units, see the launch)
+  if (bh >= a.units) return;
   const int b = bh / a.Hkv, kvh = bh % a.Hkv;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int lq = warp & 3, cg = (warp - 4) >> 2;         // (epilogue warps) lane quarter, 64-column group
@@ -872,12 +875,20 @@ cudaError_t launch_scores_t(const CUtensorMap& qm, const CUtensorMap& k256, cons
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(colsum_tc_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem2);
   if (e != cudaSuccess) return e;
+  // Large grids go through the units in groups, within a group the longest blocks of all its units first: groups
+  // of about 512 block pairs or 256 wide key blocks keep the streamed tiles of the CTAs at work in L2 (batch 8,
+  // T = 16384: 13.4-13.9 ms ungrouped, 13.0 so; batch 4, T = 8192: 1.76 and 1.73) and the last CTAs short (one
+  // unit at a time: batch 1, T = 4096 198 us, 189 so).
+  const int64_t pairs = ceil_div(a.rowblocks, 2);
   // Two row blocks per CTA from 1.5 waves of pairs: 256 pairs (16/2 heads, T = 4096) 194 -> 188 us, 188 pairs
   // (T = 3000) 151 -> 155; below, the longest CTA is the time.
-  if (a.n_ksplit == 1 && (int64_t)units * ceil_div(a.rowblocks, 2) * 2 >= 3 * kNumSMs && a.rowblocks > 1)
-    rowstats_tc_kernel<D, 2><<<dim3(units, (unsigned)ceil_div(a.rowblocks, 2)), kThr, smem1w, st>>>(qm, k256, a);
-  else
+  if (a.n_ksplit == 1 && units * pairs * 2 >= 3 * kNumSMs && a.rowblocks > 1) {
+    const int group = (int)std::min<int64_t>(units, ceil_div(512, pairs));
+    rowstats_tc_kernel<D, 2><<<dim3(group, (unsigned)pairs, (unsigned)ceil_div(units, group)), kThr, smem1w, st>>>(qm,
+                                                                                                                 k256, a);
+  } else {
     rowstats_tc_kernel<D, 1><<<dim3(a.n_ksplit, a.rowblocks, units), kThr, smem1, st>>>(qm, k256, a);
+  }
   e = cudaPeekAtLastError();
   if (e != cudaSuccess) return e;
   if (a.rowblocks == 1) {                 // one query block: hold it, stream pass 1's key splits
@@ -899,7 +910,9 @@ cudaError_t launch_scores_t(const CUtensorMap& qm, const CUtensorMap& k256, cons
     static_assert(smem3 <= 227 * 1024, "shared memory");
     e = cudaFuncSetAttribute(colsum_wide_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem3);
     if (e != cudaSuccess) return e;
-    colsum_wide_kernel<D><<<dim3(units, (unsigned)wide), kWideThr, smem3, st>>>(qm, k256, a);
+    const int group = (int)std::min<int64_t>(units, ceil_div(256, wide));
+    colsum_wide_kernel<D><<<dim3(group, (unsigned)wide, (unsigned)ceil_div(units, group)), kWideThr, smem3, st>>>(qm, k256,
+                                                                                                               a);
     return cudaPeekAtLastError();
   }
   colsum_tc_kernel<D><<<dim3(keyblocks, units), kThr, smem2, st>>>(qm, k128, a);
@@ -941,6 +954,7 @@ cudaError_t launch_prefill_scores(const mkv_config& c, const void* q, int64_t q_
   a.pos0 = T - q_rows;
   a.Hq = c.Hq;
   a.Hkv = c.Hkv;
+  a.units = c.B * c.Hkv;
   a.G = c.Hq / c.Hkv;
   a.rpb = kTM / a.G;
   a.rowblocks = (int)ceil_div(q_rows, a.rpb);
