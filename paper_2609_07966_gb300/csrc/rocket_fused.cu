@@ -47,6 +47,12 @@ namespace {
 
 constexpr int kRfWarps = 8;
 constexpr int kRfThreads = kRfWarps * 32;
+// Up to this many candidate pages are ranked by counting the pages ahead of each (one pass over them), more by
+// bits of the k-th key, a barrier a bit or, beyond 256 pages, two.  Counting against bits: 8/2 heads, D = 64,
+// batch 1, us a launch: 18 pages 8.0 -> 7.1, 62 pages 8.7 -> 7.5, 124 pages 9.4 -> 8.5.  Two bits against one:
+// 361 pages 12.0 -> 10.7, 999 pages (256 kept) 13.5 -> 12.1; up to 256 pages, where the barrier itself counts
+// a bit, two took 0.1 to 0.4 us longer.
+constexpr int kRankPages = 128;
 
 __device__ __forceinline__ uint32_t cluster_rank() {
   uint32_t r;
@@ -389,8 +395,8 @@ __global__ void __launch_bounds__(kRfThreads, 2) rocket_fused_kernel(const RfArg
         __syncthreads();
       }
 
-      // ---- 3. the k best pages under (score desc, page asc), by every CTA for itself.  The k-th largest
-      // score key bit by bit, from the highest bit in which the keys differ, the keys that reach a
+      // ---- 3. the k best pages under (score desc, page asc), by every CTA for itself.  Few pages are ranked
+      // by counting; of more, the k-th largest score key is found bit by bit, from the highest bit in which the keys differ, the keys that reach a
       // candidate counted by the barrier itself, until exactly k do or no bit is left (ties: the lower
       // pages); then the kept pages in ascending order from one word of flags per 32 pages.
       const int k = min(a.kp, ns);
@@ -409,7 +415,22 @@ __global__ void __launch_bounds__(kRfThreads, 2) rocket_fused_kernel(const RfArg
       uint32_t thr = 1;                                // kept: keys at or above it (ge),
       bool ge = true;
       int need = 0;                                    // or above it and the first `need` equal to it
-      if (k < ns) {
+      if (k < ns && ns <= kRankPages) {                // few: the pages ahead of each one counted
+        uint32_t* kp_ = reinterpret_cast<uint32_t*>(sc);
+        if (tid < ((ns + 3) & ~3)) kp_[tid] = key[0];  // (its own score; 0 behind the last)
+        __syncthreads();
+        int ahead = 0;                                 // before p: keys >= its own, after it: > its own
+        if (tid < ns) {
+          const uint32_t own = key[0], before = own - 1u;
+#pragma unroll 4
+          for (int j = 0; j < ns; j += 4) {
+            const uint4 x = *reinterpret_cast<const uint4*>(kp_ + j);
+            ahead += (x.x > (j < tid ? before : own)) + (x.y > (j + 1 < tid ? before : own)) +
+                     (x.z > (j + 2 < tid ? before : own)) + (x.w > (j + 3 < tid ? before : own));
+          }
+        }
+        key[0] = tid < ns && ahead < k ? 1u : 0u;      // (thr = 1: these are kept)
+      } else if (k < ns) {
         uint32_t mx = 0, mn = 0xffffffffu;
         for (int u = 0; u < nk; ++u) {
           const uint32_t x = key_of(u);
@@ -436,6 +457,37 @@ __global__ void __launch_bounds__(kRfThreads, 2) rocket_fused_kernel(const RfArg
           int above = 0;                               // keys above the prefix's range
           uint32_t bit = 0x80000000u >> __clz((int)(mx ^ mn));
           thr = mx & ~(2u * bit - 1u);                 // (bit 31: 2 * bit wraps to 0, thr to 0)
+          // two bits a round while three counts fit a word; the last round may have one bit (lo = 0: its
+          // first candidate is thr itself)
+          for (; nk > 1 && ns < 1024 && bit != 0u && !ge; bit >>= 2) {
+            const uint32_t lo = bit >> 1, t1 = thr | lo, t2 = thr | bit, t3 = t2 | lo;
+            uint32_t c = 0;
+#pragma unroll
+            for (int u = 0; u < KR; ++u)
+              c += (key[u] >= t1 ? 1u : 0u) + (key[u] >= t2 ? 1u << 10 : 0u) + (key[u] >= t3 ? 1u << 20 : 0u);
+            c = __reduce_add_sync(0xffffffffu, c);
+            if (lane == 0) cnt[par][warp] = (int)c;
+            __syncthreads();
+            const int4 x = *reinterpret_cast<const int4*>(cnt[par]), y = *reinterpret_cast<const int4*>(cnt[par] + 4);
+            c = (uint32_t)(((x.x + x.y) + (x.z + x.w)) + ((y.x + y.y) + (y.z + y.w)));
+            par ^= 1;
+            const int c1 = (int)(c & 1023u), c2 = (int)((c >> 10) & 1023u), c3 = (int)(c >> 20);
+            if (c3 >= k) {
+              thr = t3;
+              ge = c3 == k;
+            } else if (c2 >= k) {
+              thr = t2;
+              above = c3;
+              ge = c2 == k;
+            } else if (c1 >= k) {
+              thr = t1;
+              above = c2;
+              ge = c1 == k;
+            } else {
+              above = c1;
+            }
+          }
+          if (ge) bit = 0u;
           for (; bit != 0u; bit >>= 1) {
             const uint32_t t = thr | bit;
             int c;
@@ -468,7 +520,7 @@ __global__ void __launch_bounds__(kRfThreads, 2) rocket_fused_kernel(const RfArg
       }
       const int words = (ns + 31) / 32;                // flags of 32 pages each: kept for sure / equal to thr
       for (int u = 0; u < nk; ++u) {
-        const uint32_t x = key_of(u);
+        const uint32_t x = ns <= kRankPages ? key[0] : key_of(u);
         const uint32_t fg = __ballot_sync(0xffffffffu, ge ? x >= thr : x > thr);
         const uint32_t fe = __ballot_sync(0xffffffffu, !ge && x == thr);
         const int w = warp + u * kRfWarps;

@@ -19,6 +19,10 @@ CASES = [  # B, Hq, Hkv, D, slots held, slots, pages chosen, dims, values
     (1, 8, 1, 128, 16400, 16432, 257, 128, "ties"), (1, 8, 2, 64, 40000, 40016, 300, 3, "ties"),
     (2, 8, 2, 64, 777, 784, 48, 16, "equal"), (130, 1, 1, 64, 2000, 2000, 11, 16, "equal"),
     (1, 2, 2, 128, 1, 16, 4, 8, "plain"), (1, 4, 2, 64, 16, 32, 4, 8, "plain"), (2, 4, 2, 64, 17, 32, 1, 8, "plain"),
+    # at most 128 candidate pages counted, up to 1023 by two bits a round, more by one
+    (1, 8, 4, 64, 2064, 2080, 33, 16, "ties"), (2, 8, 8, 64, 2065, 2080, 128, 16, "ties"),
+    (1, 8, 2, 64, 16384, 16400, 200, 16, "ties"), (1, 8, 2, 128, 16385, 16400, 200, 16, "plain"),
+    (1, 8, 2, 64, 5000, 5008, 31, 16, "equal"), (3, 8, 2, 64, 2000, 2000, 124, 16, "equal"),
 ]
 
 
