@@ -396,7 +396,8 @@ __global__ void __launch_bounds__(kRfThreads, 2) rocket_fused_kernel(const RfArg
       }
 
       // ---- 3. the k best pages under (score desc, page asc), by every CTA for itself.  Few pages are ranked
-      // by counting; of more, the k-th largest score key is found bit by bit, from the highest bit in which the keys differ, the keys that reach a
+      // by counting; of more, the k-th largest score key is found bit by bit, from the highest bit in which the
+      // keys differ, the keys that reach a
       // candidate counted by the barrier itself, until exactly k do or no bit is left (ties: the lower
       // pages); then the kept pages in ascending order from one word of flags per 32 pages.
       const int k = min(a.kp, ns);
