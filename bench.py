@@ -341,7 +341,8 @@ class Runner:
             # (layers 0 and 1 follow the previous step's updates, joined at its end)
             torch.cuda.current_stream().wait_event(self.upd_ev[l % 2])
         if self.method in ("fp16", "h2o", "kvquant") and self.step_fused:
-            # append (KVQuant: quantize) and attention in one launch, then (H2O) the update
+            # append and attention in one launch (KVQuant: quantize with attention starting beneath it, two
+            # launches in one call), then (H2O) the update
             kn = self.kn[l] if kn is None else kn
             vn = self.vn[l] if vn is None else vn
             q = self.q[l] if q is None else q
@@ -407,8 +408,8 @@ class Runner:
             self.step()
 
     def launches_per_step(self):
-        # per layer: FP16 / H2O / KVQuant append (KVQuant: quantize) and attention in one launch (H2O:
-        # + score update); RocketKV append, page choice and attention in one launch
+        # per layer: FP16 / H2O append and attention in one launch (H2O: + score update); KVQuant quantize and
+        # attention; RocketKV append, page choice and attention in one launch
         per = {"fp16": 1 if self.step_fused else 2, "kvquant": 2,
                "h2o": 2 if self.step_fused else 3,
                "rocket": 1 if self.rocket_fused else 3}[self.method]
