@@ -49,7 +49,8 @@ constexpr int kRfWarps = 8;
 constexpr int kRfThreads = kRfWarps * 32;
 // Up to this many candidate pages are ranked by counting the pages ahead of each (one pass over them), more by
 // bits of the k-th key, a barrier a bit or, beyond 256 pages, two.  Counting against bits: 8/2 heads, D = 64,
-// batch 1, us a launch: 18 pages 8.0 -> 7.1, 62 pages 8.7 -> 7.5, 124 pages 9.4 -> 8.5.  Two bits against one:
+// batch 1, us a launch: 18 pages 8.0 -> 7.1, 62 pages 8.7 -> 7.5, 124 pages 9.4 -> 8.5, 156
+// pages 9.3 both, 256 pages (64 kept) 9.2 -> 10.1.  Two bits against one:
 // 361 pages 12.0 -> 10.7, 999 pages (256 kept) 13.5 -> 12.1; up to 256 pages, where the barrier itself counts
 // a bit, two took 0.1 to 0.4 us longer.
 constexpr int kRankPages = 128;
