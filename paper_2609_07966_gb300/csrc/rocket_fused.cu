@@ -189,9 +189,9 @@ __global__ void __launch_bounds__(kRfThreads, 2) rocket_fused_kernel(const RfArg
   const int b = (int)(bh / a.Hkv), kvh = (int)(bh % a.Hkv);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int g = lane >> 2, r = lane & 3;
-  // this CTA's share of the pages, fixed by the capacity so the prefetch need not wait for T_len
+  // this CTA's share of the pages, by the capacity
   const int sp = (int)((a.npc + CL - 1) / CL);          // pages per CTA
-  const int p0 = min((int)a.npc, rank * sp), npf = min((int)a.npc, p0 + sp) - p0;
+  const int p0 = min((int)a.npc, rank * sp);
 
   // the group's query (fp16) and the cache length
   constexpr int kQW = (8 * D / 2 + kRfThreads - 1) / kRfThreads;   // query words per thread (G <= 8)
@@ -255,14 +255,16 @@ __global__ void __launch_bounds__(kRfThreads, 2) rocket_fused_kernel(const RfArg
     if (i < D && half == 0 && rk < a.rd) dims[rk] = i;
   }
   __syncthreads();
-  // ---- 1. the chosen dims' bounds of this CTA's pages, row t for the t-th dim (16-byte copies from
-  // the row start rounded down to 16 bytes, the last one cut at the end of the pages)
+  // ---- 1. the chosen dims' bounds of this CTA's candidate pages, row t for the t-th dim (16-byte copies
+  // from the row start rounded down to 16 bytes, the last one cut at the end of the pages).  With no candidate
+  // page nothing is copied: CTA 0's bounds are also where it receives the cluster's partials, and only its
+  // scores tell the other CTAs that its copies have landed.
   for (int row = tid >> 3; row < 2 * a.rd; row += kRfThreads / 8) {   // eight threads per row
     const int which = row >= a.rd ? 1 : 0, t = which ? row - a.rd : row;
     const int64_t start = (bh * D + dims[t]) * a.npc + p0;
     const __half* src = (which ? a.kmax : a.kmin) + (start & ~7ll);
     __half* dst = (which ? bmx : bmn) + t * a.rs;
-    const int off = (int)(start & 7), left = npf > 0 ? off + npf : 0;   // halves from the first copy's start
+    const int off = (int)(start & 7), left = np > 0 ? off + np : 0;   // halves from the first copy's start
     if (which == 0 && (tid & 7) == 0) boff[t] = t * a.rs + off;
     for (int h = (tid & 7) * 8; h < left; h += 64) cp_async16(dst + h, src + h, min(16, (left - h) * 2));
   }

@@ -57,3 +57,37 @@ def test_fused_equals_two_calls(B, Hq, Hkv, D, n, cap, pages, dims, values):
     assert torch.equal(idx, idx2)
     assert_close(out2.float().cpu(), out.float().cpu(), "fused against two calls")
     assert mkv.mkv_get_status() == 0
+
+
+@pytest.mark.parametrize("Hkv,D,T_cap,dims", [(4, 64, 32, 32), (4, 64, 4160, 32), (2, 128, 8192, 128), (25, 64, 4160, 32),
+                                              (16, 64, 4160, 64)])
+def test_no_candidate_page(Hkv, D, T_cap, dims):
+    """At most 16 tokens in a cache of any capacity (one head a group, so that the page bounds of the capacity are
+    larger than a CTA's partial): the newest page is the whole result, in every call the same bits."""
+    torch = torch_cuda()
+    dev = torch.device("cuda")
+    lens = [1, 2, 15, 16]
+    B, reps = len(lens), 50
+    g = torch.Generator(device=dev).manual_seed(T_cap + Hkv)
+    cfg = mkv.config(mkv.MKV_ROCKET, B, Hkv, Hkv, D, snap_window=1, snap_keep=T_cap, topk_pages=3, topq_dims=dims)
+    c = caches.alloc_cache(cfg, T_cap, device=dev)
+    for name in ("k", "v", "kmin", "kmax"):            # (bounds of pages that do not exist: never looked at)
+        c.t[name].normal_(generator=g)
+    q = torch.randn((B, Hkv, D), device=dev, generator=g).half()
+    n = torch.tensor(lens, dtype=torch.int32, device=dev)
+    c.t["T_len"].copy_(n)
+    k, v = (c.t[x][:, :, :16].double() for x in ("k", "v"))
+    s = torch.einsum("bhd,bhtd->bht", q.double(), k) / D ** 0.5
+    s = s.masked_fill(torch.arange(16, device=dev) >= n[:, None, None], float("-inf"))
+    ref = torch.einsum("bht,bhtd->bhd", torch.softmax(s, -1), v)
+    idx = torch.full((reps, B, Hkv, 3), -7, dtype=torch.int32, device=dev)
+    out = torch.full((2 * reps, B, Hkv, D), float("nan"), dtype=torch.float16, device=dev)
+    for i in range(reps):
+        mkv.mkv_rocket_decode(cfg, q.data_ptr(), c.c, idx[i].data_ptr(), out[i].data_ptr())
+    kn, vn = (torch.stack([c.t[x][b, :, lens[b] - 1] for b in range(B)]) for x in ("k", "v"))
+    for i in range(reps):                              # the same with the last token appended by the step
+        c.t["T_len"].copy_(n - 1)
+        mkv.mkv_rocket_step(cfg, q.data_ptr(), kn.data_ptr(), vn.data_ptr(), c.c, 0, out[reps + i].data_ptr())
+    assert mkv.mkv_get_status() == 0 and torch.equal(c.t["T_len"], n) and bool((idx == -1).all())
+    assert_close(out[0].double().cpu(), ref.cpu(), "newest page alone")
+    assert bool((out == out[0]).all())
