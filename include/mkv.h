@@ -403,7 +403,7 @@ mkv_status mkv_rocket_select(const mkv_config* cfg, const void* q, const mkv_cac
  * NULL to skip) int32 [B][Hkv][topk_pages] as mkv_rocket_select writes it.
  * The page scores are the same sums in another fp32 order, so a near-tie
  * may pick another page than mkv_rocket_select.  MKV_ERR_UNSUPPORTED when
- * T_cap is too long for the step's shared memory (about 32K slots at D=128);
+ * T_cap is too long for the step's shared memory (about 32K slots at D=128, whatever B, Hkv and topq_dims);
  * use the two calls then. */
 mkv_status mkv_rocket_decode(const mkv_config* cfg, const void* q, const mkv_cache* cache,
                              int32_t* page_idx_out, void* out, void* stream);

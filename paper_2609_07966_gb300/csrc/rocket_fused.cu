@@ -777,11 +777,17 @@ __global__ void __launch_bounds__(kRfThreads, 2) rocket_fused_kernel(const RfArg
   }
 }
 
+constexpr int kRfDynMax = (227 - 5) * 1024;   // dynamic shared memory beside the kernel's 4.8 KB of static
+
+int rf_row(int64_t npc, int cl) { return ((int)((npc + cl - 1) / cl) + 8 + 7) / 8 * 8; }   // halves per bounds row
+size_t rf_smem(const RfArgs& a, int D, int cl) {
+  return (size_t)RfLayout(D, a.G, a.npc, a.kp, a.rd, rf_row(a.npc, cl), cl).bytes;
+}
+
 template <int D, int CL>
 cudaError_t launch_rf_t(RfArgs a, int units, cudaStream_t st) {
-  const int sp = (int)((a.npc + CL - 1) / CL);
-  a.rs = (sp + 8 + 7) / 8 * 8;
-  const size_t smem = (size_t)RfLayout(D, a.G, a.npc, a.kp, a.rd, a.rs, CL).bytes;
+  a.rs = rf_row(a.npc, CL);
+  const size_t smem = rf_smem(a, D, CL);
   cudaError_t e = cudaFuncSetAttribute(rocket_fused_kernel<D, CL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   cudaLaunchAttribute attr[1];
@@ -806,18 +812,24 @@ cudaError_t launch_rf_t(RfArgs a, int units, cudaStream_t st) {
 //   32 units 14.0 / 13.5 / 16.5 / 20.2; 24.6 / 25.1 / 39.4 / 54.1
 //   64 units 26.1 / 17.0 / 17.5 / 20.6; 49.5 / 36.6 / 43.2 / 57.1
 //  128 units 49.0 / 32.0 / 23.2 / 22.3; 96.3 / 73.3 / 64.6 / 59.7
+// A CTA holds the chosen dims' bounds and the partial scores of its 1 / CL of the pages, so long caches and many
+// dims need more CTAs than that (32/8 heads, D = 128, 128 units: 20160 slots fit CL = 1 with 32 dims, 5888
+// with 128); eight hold every accepted length.
 template <int D>
 cudaError_t launch_rf_d(const RfArgs& a, int units, cudaStream_t st) {
-  if (units <= 16) return launch_rf_t<D, 8>(a, units, st);
-  if (units <= 64) return launch_rf_t<D, 4>(a, units, st);
-  if (units <= 112) return launch_rf_t<D, 2>(a, units, st);
+  int cl = units <= 16 ? 8 : units <= 64 ? 4 : units <= 112 ? 2 : 1;
+  while (cl < kRocketCluster && rf_smem(a, D, cl) > (size_t)kRfDynMax) cl *= 2;
+  if (cl == 8) return launch_rf_t<D, 8>(a, units, st);
+  if (cl == 4) return launch_rf_t<D, 4>(a, units, st);
+  if (cl == 2) return launch_rf_t<D, 2>(a, units, st);
   return launch_rf_t<D, 1>(a, units, st);
 }
 
 }  // namespace
 
-// Bytes that bound the accepted cache length: the page scores, the kept flags and every dim's bounds of
-// an eighth of the pages (the layout behind the documented limit; the kernel's own, RfLayout, is smaller)
+// Bytes that bound the accepted cache length: the page scores, the kept flags, every dim's bounds of an eighth
+// of the pages and the warps' staged pages (the layout behind the documented limit).  RfLayout for eight CTAs
+// needs at most 209104 bytes for a length within it.
 size_t rocket_fused_smem(const mkv_config& c, int64_t T_cap) {
   const int D = c.D, G = c.Hq / c.Hkv, kp = c.topk_pages;
   const int64_t npc = T_cap / kPage;

@@ -91,3 +91,46 @@ def test_no_candidate_page(Hkv, D, T_cap, dims):
     assert mkv.mkv_get_status() == 0 and torch.equal(c.t["T_len"], n) and bool((idx == -1).all())
     assert_close(out[0].double().cpu(), ref.cpu(), "newest page alone")
     assert bool((out == out[0]).all())
+
+
+# units at each preferred cluster size, with the longest cache the step accepts: where the bounds and partial scores
+# of a CTA's pages do not fit, more CTAs share a unit
+@pytest.mark.parametrize("B,Hkv,D,dims", [(2, 8, 128, 128), (4, 8, 128, 128), (4, 16, 128, 32), (16, 4, 128, 128), (7, 16, 128, 64),
+                                          (8, 16, 128, 32), (8, 16, 128, 128), (32, 8, 128, 64), (8, 16, 64, 16), (14, 8, 64, 64)])
+def test_longest_accepted_cache(B, Hkv, D, dims):
+    torch = torch_cuda()
+    dev = torch.device("cuda")
+    T_cap, G, pages, steps = 32768 if D == 128 else 65536, 4 if D == 128 else 2, 9, 3
+    g = torch.Generator(device=dev).manual_seed(B * Hkv + dims)
+    cfg = mkv.config(mkv.MKV_ROCKET, B, G * Hkv, Hkv, D, snap_window=1, snap_keep=T_cap, topk_pages=pages, topq_dims=dims)
+    twins = [caches.alloc_cache(cfg, T_cap, device=dev) for _ in range(2)]
+    a, c = twins
+    for name in ("k", "v"):                            # integers: page scores are exact in any order
+        a.t[name].copy_(torch.randint(-9, 10, a.t[name].shape, generator=g, device=dev, dtype=torch.int8))
+        a.t[name].div_(8)
+    pg = a.t["k"].unflatten(2, (T_cap // 16, 16))
+    a.t["kmin"].copy_(pg.amin(3).transpose(2, 3))
+    a.t["kmax"].copy_(pg.amax(3).transpose(2, 3))
+    a.t["T_len"].fill_(T_cap - 2)                      # the last step finds the cache full
+    a.t["T_len"][0] = 5000
+    for name in a.t:
+        c.t[name].copy_(a.t[name])
+    ws, nws = caches.workspace(cfg, T_cap, device=dev)
+    for s in range(steps):
+        q = torch.randint(-3, 4, (B, G * Hkv, D), generator=g, device=dev).half() / 4
+        kn, vn = (torch.randint(-9, 10, (B, Hkv, D), generator=g, device=dev).half() / 8 for _ in range(2))
+        idx, idx1 = (torch.full((B, Hkv, pages), -7, dtype=torch.int32, device=dev) for _ in range(2))
+        ref, out, out1 = torch.empty_like(q), torch.empty_like(q), torch.empty_like(q)
+        full = (0, mkv.MKV_FLAG_CACHE_FULL)[s == steps - 1]
+        mkv.mkv_append_kv(cfg, kn.data_ptr(), vn.data_ptr(), a.c)
+        assert mkv.mkv_get_status() == full
+        mkv.mkv_rocket_select(cfg, q.data_ptr(), a.c, idx.data_ptr())
+        mkv.mkv_decode_attention(cfg, q.data_ptr(), a.c, None, idx.data_ptr(), ref.data_ptr(), ws.data_ptr(), nws)
+        mkv.mkv_rocket_decode(cfg, q.data_ptr(), a.c, idx1.data_ptr(), out1.data_ptr())
+        assert torch.equal(idx, idx1)
+        mkv.mkv_rocket_step(cfg, q.data_ptr(), kn.data_ptr(), vn.data_ptr(), c.c, idx1.fill_(-7).data_ptr(), out.data_ptr())
+        assert mkv.mkv_get_status() == full
+        assert torch.equal(idx, idx1) and torch.equal(out, out1)
+        assert_close(out.float().cpu(), ref.float().cpu(), f"step {s}")
+        for name in a.t:
+            assert torch.equal(a.t[name], c.t[name]), (s, name)
