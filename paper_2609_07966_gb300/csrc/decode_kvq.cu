@@ -40,7 +40,13 @@
 // mkv_kvquant_step launches the quantize kernel and then this one with the programmatic
 // stream-serialization attribute: its CTAs start while the token is being quantized, load the rotation
 // table, the first unit's tables and the query, and wait (griddepcontrol.wait) before they read the cache.
-// (Only there: a predecessor that this call did not launch could still be writing the query.)
+// (Only there: a predecessor that this call did not launch could still be writing the query.  The quantize
+// kernel lets this one start only after its own wait, so all that was launched before it has completed.)
+// What the quantize kernel writes is not constant while this one runs: it is read after the wait by cp.async, plain
+// loads or __ldcg, never through the read-only path (__ldg), which is for the tables.  (ptxas schedules the loops
+// around these few loads differently: as they are, a pass of two 8 x 8K layers at 4 bits takes 215.1 us, of one 128K
+// layer at 2 bits 177.7, of one 32 x 4K layer at 3 bits 194.9; with __ldg 215.2, 177.7 and 194.9, with the entries
+// by __ldcg too 219.0, 177.8 and 202.8.)
 // Quantizing the token inside this launch, by the attention warps of the CTA that holds its chunk, was
 // slower at every size measured (B = 8, 8K, 4 bits: 106.4 us a step in a graph against 101.4 for two plain
 // launches; 2 x 3000: 27.4 against 26.8): the attention's first chunks waited for it.
@@ -474,8 +480,8 @@ __global__ void __launch_bounds__(kThr, 1) decode_kvq_kernel(const KvqArgs a) {
       if (s < nchunks) {
         load_chunk(s, s);
         if (s == 0 && ptid < kEnt) {
-          const int e0 = __ldg(a.k_out_off + off_base + v_begin);
-          const int e1 = min(__ldg(a.k_out_off + off_base + min(v_begin + kChunk, (int64_t)n_len)),
+          const int e0 = __ldcg(a.k_out_off + off_base + v_begin);
+          const int e1 = min(__ldcg(a.k_out_off + off_base + min(v_begin + kChunk, (int64_t)n_len)),
                              (int)a.k_out_cap);
           load_entries(0, e0, e1);
         }
@@ -634,7 +640,7 @@ __global__ void __launch_bounds__(kThr, 1) decode_kvq_kernel(const KvqArgs a) {
         auto fetch = [&](int e) -> uint32_t {
           if (e < 0 || e >= e_hi) return 0xffff0000u;  // no entry: not a channel
           if (e - E0 < kEnt) return ents[e - E0];
-          return __ldg(gents + e);  // beyond the staged entries
+          return gents[e];  // beyond the staged entries
         };
         auto fix = [&](uint32_t ev, int pass) {
           const int ch = (int)((ev >> 16) & 0xffu);
@@ -674,7 +680,7 @@ __global__ void __launch_bounds__(kThr, 1) decode_kvq_kernel(const KvqArgs a) {
           const int t = t0w + (e & 15), k = e >> 4;
           if (t0 + t >= n_len) continue;
           const uint32_t ev = a.n_v <= Lay::NVS ? reinterpret_cast<const uint32_t*>(B_ + Lay::B_VO)[k * kChunk + t]
-                                                : __ldg(a.v_out + (bh * a.T_cap + t0 + t) * a.n_v + k);
+                                                : a.v_out[(bh * a.T_cap + t0 + t) * a.n_v + k];
           const int chn = (int)(ev >> 16);
           if (chn >= D) continue;
           const int col = chn < NP ? 2 * chn : 2 * (chn - NP) + 1;
