@@ -17,7 +17,8 @@
  *    device memory; scratch space is the caller's `ws` buffer, sized by
  *    mkv_workspace_size().  The first 16 KiB of a workspace hold counters
  *    that must be zero before the first call that uses it (allocate it
- *    zero-filled); every call leaves them zero again.  Calls that share a
+ *    zero-filled); every call leaves them zero again.  It starts at a
+ *    multiple of 4 bytes (16: a little faster).  Calls that share a
  *    workspace must not overlap on the GPU.  Nothing is retained between
  *    calls except the library's status word (see mkv_get_status).
  *  - B * Hkv is at most 4096.

@@ -78,6 +78,21 @@ __device__ __forceinline__ uint32_t pack_half2(float lo, float hi) {
   return *reinterpret_cast<uint32_t*>(&h);
 }
 
+// Two and four neighbouring results, rounded to fp16, at an even index of an output row: together where the caller's
+// pointer is 4-byte aligned (it only has to be an fp16 pointer).
+__device__ __forceinline__ void store_out2(__half* p, float x, float y) {
+  if ((reinterpret_cast<uintptr_t>(p) & 3) == 0) {
+    *reinterpret_cast<__half2*>(p) = __floats2half2_rn(x, y);
+  } else {
+    p[0] = __float2half_rn(x);
+    p[1] = __float2half_rn(y);
+  }
+}
+__device__ __forceinline__ void store_out4(__half* p, float x, float y, float z, float w) {
+  store_out2(p, x, y);
+  store_out2(p + 2, z, w);
+}
+
 // Exact fp16 -> fp32 widening of raw bits.
 __device__ __forceinline__ float h2f(uint16_t bits) { return __half2float(__ushort_as_half(bits)); }
 

@@ -44,7 +44,8 @@ __device__ __forceinline__ void merge_if_last(const MergeArgs& a, int64_t bh, in
   __threadfence();
   const int ns = n_parts > 0 ? n_parts : a.n_split, stride = a.n_split, G = a.G;
   const int64_t hq0 = (int64_t)b * a.Hq + (int64_t)kvh * G;
-  if (2 * G * ns + 2 * G + 4 * NT + 4 <= cap) {
+  // (a workspace that is not 16-byte aligned takes the direct loop below)
+  if (2 * G * ns + 2 * G + 4 * NT + 4 <= cap && (reinterpret_cast<uintptr_t>(a.part_o) & 15) == 0) {
     const int quads = G * (D / 4);               // (head, four dims)
     const int SL = quads < NT ? NT / quads : 1;  // slices of the splits per quad
     float* f = scratch;                          // [G][ns] m, then the weights 2^(m_s - M)
@@ -127,9 +128,8 @@ __device__ __forceinline__ void merge_if_last(const MergeArgs& a, int64_t bh, in
       if (sl == 0) {
         const int row = quad / (D / 4), d = quad % (D / 4) * 4;
         const float L = tot[G + row];
-        __half2* out = reinterpret_cast<__half2*>(a.out + (hq0 + row) * D + d);
-        out[0] = __floats2half2_rn(L > 0.f ? O.x / L : 0.f, L > 0.f ? O.y / L : 0.f);
-        out[1] = __floats2half2_rn(L > 0.f ? O.z / L : 0.f, L > 0.f ? O.w / L : 0.f);
+        store_out4(a.out + (hq0 + row) * D + d, L > 0.f ? O.x / L : 0.f, L > 0.f ? O.y / L : 0.f,
+                   L > 0.f ? O.z / L : 0.f, L > 0.f ? O.w / L : 0.f);
         if (a.m_tot != nullptr && d == 0) {
           a.m_tot[hq0 + row] = tot[row];
           a.l_tot[hq0 + row] = L;

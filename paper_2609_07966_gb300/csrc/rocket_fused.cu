@@ -717,9 +717,7 @@ __global__ void __launch_bounds__(kRfThreads, 2) rocket_fused_kernel(const RfArg
       }
     } else {
       const float inv = Lsum > 0.f ? 1.f / Lsum : 0.f;
-      __half2* out = reinterpret_cast<__half2*>(a.out + ((int64_t)b * a.Hq + (int64_t)kvh * G + row) * D + d);
-      out[0] = __floats2half2_rn(O.x * inv, O.y * inv);
-      out[1] = __floats2half2_rn(O.z * inv, O.w * inv);
+      store_out4(a.out + ((int64_t)b * a.Hq + (int64_t)kvh * G + row) * D + d, O.x * inv, O.y * inv, O.z * inv, O.w * inv);
     }
   }
   if constexpr (CL > 1) {
@@ -744,8 +742,7 @@ __global__ void __launch_bounds__(kRfThreads, 2) rocket_fused_kernel(const RfArg
           }
         }
         const float inv = Lsum > 0.f ? 1.f / Lsum : 0.f;
-        *reinterpret_cast<__half2*>(a.out + ((int64_t)b * a.Hq + (int64_t)kvh * G + row) * D + d) =
-            __floats2half2_rn(O.x * inv, O.y * inv);
+        store_out2(a.out + ((int64_t)b * a.Hq + (int64_t)kvh * G + row) * D + d, O.x * inv, O.y * inv);
       }
     }
   }
