@@ -18,7 +18,9 @@
  *    mkv_workspace_size().  The first 16 KiB of a workspace hold counters
  *    that must be zero before the first call that uses it (allocate it
  *    zero-filled); every call leaves them zero again.  It starts at a
- *    multiple of 4 bytes (16: a little faster).  Calls that share a
+ *    multiple of 4 bytes (16: a little faster); of 16 in mkv_h2o_update with
+ *    Hq / Hkv = 4 and in prompt scoring of more than 128 / (Hq / Hkv) query
+ *    rows, of 8 in any prompt scoring (else MKV_ERR_INVALID_ARG).  Calls that share a
  *    workspace must not overlap on the GPU.  Nothing is retained between
  *    calls except the library's status word (see mkv_get_status).
  *  - B * Hkv is at most 4096.

@@ -261,6 +261,14 @@ mkv_status check_qparams(const mkv_config* c, const mkv_quant_params* p, bool ne
     if (s_ != MKV_OK) return s_;   \
   } while (0)
 
+// Prompt scoring over `rows` query rows keeps (m, l) pairs in the workspace; of more than one 128-row query block
+// it copies them in bulk.
+mkv_status check_score_ws(const mkv_config* c, int64_t rows, const void* ws) {
+  const unsigned need = rows > 128 / (c->Hq / c->Hkv) ? 16 : 8;
+  MKV_REQUIRE((uintptr_t)ws % need == 0, MKV_ERR_INVALID_ARG, "the workspace of this prompt must be %u-byte aligned", need);
+  return MKV_OK;
+}
+
 size_t workspace_bytes(const mkv_config* c, int64_t T_cap) {
   size_t b = decode_ws(*c, T_cap, decode_split(*c, T_cap), nullptr).bytes;
   if (c->method == MKV_H2O || c->method == MKV_ROCKET) b = std::max(b, prefill_ws(*c, T_cap, nullptr).bytes);
@@ -504,6 +512,7 @@ mkv_status mkv_h2o_prefill(const mkv_config* cfg, const void* q_prompt, const vo
   const PrefillWs need = prefill_ws(*cfg, T, nullptr);
   MKV_REQUIRE(ws != nullptr && ws_bytes >= need.bytes, MKV_ERR_WORKSPACE,
               "workspace %zu bytes < %zu needed", ws_bytes, need.bytes);
+  MKV_TRY(check_score_ws(cfg, T, ws));
   const PrefillWs w = prefill_ws(*cfg, T, ws);
   cudaStream_t st = as_stream(stream);
   MKV_CUDA(launch_prefill_scores(*cfg, q_prompt, T, T, full_k, w, st));
@@ -519,6 +528,8 @@ mkv_status mkv_h2o_update(const mkv_config* cfg, mkv_cache* cache, void* ws, siz
   const DecodeWs need = decode_ws(*cfg, cache->T_cap, sp, nullptr);
   MKV_REQUIRE(ws != nullptr && ws_bytes >= need.bytes, MKV_ERR_WORKSPACE,
               "workspace %zu bytes < %zu needed", ws_bytes, need.bytes);
+  MKV_REQUIRE(cfg->Hq / cfg->Hkv != 4 || (uintptr_t)ws % 16 == 0, MKV_ERR_INVALID_ARG,
+              "the workspace of h2o_update must be 16-byte aligned with 4 heads a group (their logits are read together)");
   MKV_CUDA(launch_h2o_update(*cfg, *cache, decode_ws(*cfg, cache->T_cap, sp, ws), as_stream(stream)));
   return MKV_OK;
 }
@@ -538,6 +549,7 @@ mkv_status mkv_snap_compress(const mkv_config* cfg, const void* q_window, const 
   const PrefillWs need = prefill_ws(*cfg, T, nullptr);
   MKV_REQUIRE(ws != nullptr && ws_bytes >= need.bytes, MKV_ERR_WORKSPACE,
               "workspace %zu bytes < %zu needed", ws_bytes, need.bytes);
+  if (T > cfg->snap_keep) MKV_TRY(check_score_ws(cfg, cfg->snap_window, ws));
   const PrefillWs w = prefill_ws(*cfg, T, ws);
   cudaStream_t st = as_stream(stream);
   if (T > cfg->snap_keep) MKV_CUDA(launch_prefill_scores(*cfg, q_window, cfg->snap_window, T, full_k, w, st));

@@ -213,3 +213,21 @@ def test_kvquant_step_accepts_the_tested_shapes(L):
         st = L.mkv_kvquant_step(ctypes.byref(kq), ctypes.byref(qp), 64, 80, 96, ctypes.byref(cache), 128, 4096,
                                 ctypes.c_size_t(1 << 40), None)
         assert st == mkv.MKV_ERR_CUDA, (B, Hkv, T_cap, st, mkv.mkv_last_error())
+
+
+def test_workspace_alignment_is_checked_where_it_is_needed(L):
+    """A workspace that a call's wide loads could not be made from is refused on the host."""
+    cache = mkv.mkv_cache()
+    cache.T_cap, cache.T_len, cache.k, cache.v = 1024, 8, 256, 512
+    cache.pos, cache.acc, cache.slot, cache.kmin, cache.kmax = 768, 1024, 1280, 1536, 1792
+    cfg = mkv.config(mkv.MKV_H2O, 1, 8, 2, 64, h2o_heavy=100, h2o_recent=100)
+    for at in (4096 + 8, 4096 + 4):                          # 4 heads a group: four logits a load
+        st = L.mkv_h2o_update(ctypes.byref(cfg), ctypes.byref(cache), at, 1 << 40, None)
+        assert st == mkv.MKV_ERR_INVALID_ARG and "16-byte aligned" in mkv.mkv_last_error()
+    for T, at, need in ((33, 4096 + 8, 16), (32, 4096 + 4, 8)):
+        st = L.mkv_h2o_prefill(ctypes.byref(cfg), 64, 64, 64, T, ctypes.byref(cache), at, 1 << 40, None)
+        assert st == mkv.MKV_ERR_INVALID_ARG and f"{need}-byte aligned" in mkv.mkv_last_error()
+    for W, at, need in ((33, 4096 + 8, 16), (32, 4096 + 4, 8)):
+        rc = mkv.config(mkv.MKV_ROCKET, 1, 8, 2, 64, snap_window=W, snap_pool=7, snap_keep=256, topk_pages=4, topq_dims=16)
+        st = L.mkv_snap_compress(ctypes.byref(rc), 64, 64, 64, 1000, ctypes.byref(cache), None, at, 1 << 40, None)
+        assert st == mkv.MKV_ERR_INVALID_ARG and f"{need}-byte aligned" in mkv.mkv_last_error()
