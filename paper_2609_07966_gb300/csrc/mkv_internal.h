@@ -6,6 +6,7 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <utility>
 
 #include "mkv.h"
@@ -78,6 +79,22 @@ CalibWs calib_ws(const mkv_config& c, int64_t N, void* base);
 
 struct MergeArgs;
 MergeArgs merge_args(const mkv_config& c, const DecodeWs& ws, const Split& sp, void* out, bool h2o_stats);
+
+// Lets launches of kKernel take all the shared memory of a CTA (227 KB) beside its static one.  The limit belongs to the
+// function, not to a launch: one that followed each call's size could undercut another host thread's between
+// its setting and its launch.
+template <auto kKernel>
+cudaError_t allow_all_smem() {
+  static std::atomic<int> most{-1};       // (the same on every device)
+  int m = most.load(std::memory_order_relaxed);
+  if (m < 0) {
+    cudaFuncAttributes at;
+    const cudaError_t e = cudaFuncGetAttributes(&at, kKernel);
+    if (e != cudaSuccess) return e;
+    most.store(m = 227 * 1024 - (int)at.sharedSizeBytes, std::memory_order_relaxed);
+  }
+  return cudaFuncSetAttribute(kKernel, cudaFuncAttributeMaxDynamicSharedMemorySize, m);
+}
 
 // Launch of a decode-step kernel with the programmatic stream-serialization attribute (the kernel
 // calls pdl_wait_and_trigger() before its first global access).

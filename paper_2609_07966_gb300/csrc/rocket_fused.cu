@@ -785,7 +785,7 @@ template <int D, int CL>
 cudaError_t launch_rf_t(RfArgs a, int units, cudaStream_t st) {
   a.rs = rf_row(a.npc, CL);
   const size_t smem = rf_smem(a, D, CL);
-  cudaError_t e = cudaFuncSetAttribute(rocket_fused_kernel<D, CL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_all_smem<rocket_fused_kernel<D, CL>>();
   if (e != cudaSuccess) return e;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;

@@ -546,7 +546,7 @@ cudaError_t launch_snap_keep(const mkv_config& c, const void* full_k, const void
     const int64_t bytes = (2 * per + 2 * (c.snap_pool / 2)) * (int64_t)sizeof(float);
     a.in_smem = bytes <= kKeepSmem;
     const int smem = a.in_smem ? (int)bytes : 0;
-    cudaError_t ea = cudaFuncSetAttribute(snap_keep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t ea = allow_all_smem<snap_keep_kernel>();
     if (ea != cudaSuccess) return ea;
     snap_keep_kernel<<<dim3(kKeepCl, units), kKeepThreads, smem, st>>>(a);
     cudaError_t e = cudaPeekAtLastError();
@@ -567,7 +567,7 @@ cudaError_t launch_rocket_select(const mkv_config& c, const void* q, const mkv_c
   const int64_t npc = cache.T_cap / kPage;
   const size_t smem = ((size_t)G * c.D + ((npc + 3) & ~3ll) + 4 * kSelPages) * sizeof(float) +
                       std::max<size_t>(2 * (size_t)c.D * kSelRow * 2, 2 * (size_t)c.topq_dims * 256 * 2);
-  cudaError_t e = cudaFuncSetAttribute(rocket_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_all_smem<rocket_select_kernel>();
   if (e != cudaSuccess) return e;
   rocket_select_kernel<<<c.B * c.Hkv, kSelThreads, smem, st>>>(
       static_cast<const __half*>(q), static_cast<const __half*>(cache.kmin), static_cast<const __half*>(cache.kmax),
