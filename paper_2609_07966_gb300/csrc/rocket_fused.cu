@@ -238,17 +238,17 @@ __global__ void __launch_bounds__(kRfThreads, 2) rocket_fused_kernel(const RfArg
   __syncthreads();
   {
     // rank under (sum |q| desc, dim asc): two threads per dim, half the dims each, four at a time; dims
-    // before i count when >= a_i, that is > the float below it (a_i >= 0), dims after it when > a_i
+    // before i count when >= a_i, that is > a_i - 1, dims after it when > a_i.  The sums' bits are ranked (in the order
+    // of the values, since none is negative; a NaN comes first): every rank is taken once whatever the query holds.
     const int i = tid >> 1, half = tid & 1;
     int rk = 0;
     if (i < D) {
-      const float ai = a_dim[i];
-      const float below = ai > 0.f ? __uint_as_float(__float_as_uint(ai) - 1u) : -1.f;
+      const int ai = __float_as_int(a_dim[i]), below = ai - 1;
 #pragma unroll 8
       for (int j = half * (D / 2); j < (half + 1) * (D / 2); j += 4) {
-        const float4 v = *reinterpret_cast<const float4*>(a_dim + j);
-        const float4 c = {j < i ? below : ai, j + 1 < i ? below : ai, j + 2 < i ? below : ai, j + 3 < i ? below : ai};
-        rk += (v.x > c.x) + (v.y > c.y) + (v.z > c.z) + (v.w > c.w);
+        const int4 v = *reinterpret_cast<const int4*>(a_dim + j);
+        rk += (v.x > (j < i ? below : ai)) + (v.y > (j + 1 < i ? below : ai)) + (v.z > (j + 2 < i ? below : ai)) +
+              (v.w > (j + 3 < i ? below : ai));
       }
     }
     rk += __shfl_xor_sync(0xffffffffu, rk, 1);

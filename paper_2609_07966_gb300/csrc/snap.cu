@@ -407,13 +407,13 @@ __global__ void __launch_bounds__(kSelThreads) rocket_select_kernel(const __half
   __syncthreads();
   if (threadIdx.x < D) {
     // rank under (sum |q| desc, dim asc): four dims per shared-memory read, unrolled so the
-    // reads overlap
+    // reads overlap; the sums' bits, as in rocket_fused_kernel: every rank is taken once, with NaNs too
     const int i = threadIdx.x;
-    const float ai = a_dim[i];
+    const int ai = __float_as_int(a_dim[i]);
     int rank = 0;
 #pragma unroll 4
     for (int j = 0; j < D; j += 4) {
-      const float4 v = *reinterpret_cast<const float4*>(a_dim + j);
+      const int4 v = *reinterpret_cast<const int4*>(a_dim + j);
       rank += (v.x > ai || (v.x == ai && j < i)) + (v.y > ai || (v.y == ai && j + 1 < i)) +
               (v.z > ai || (v.z == ai && j + 2 < i)) + (v.w > ai || (v.w == ai && j + 3 < i));
     }
@@ -452,8 +452,6 @@ __global__ void __launch_bounds__(kSelThreads) rocket_select_kernel(const __half
     if (threadIdx.x < ns)
       ssc[threadIdx.x] = (part[threadIdx.x] + part[kSelPages + threadIdx.x]) +
                          (part[2 * kSelPages + threadIdx.x] + part[3 * kSelPages + threadIdx.x]);
-    else if (threadIdx.x < ((ns + 3) & ~3))
-      ssc[threadIdx.x] = -INFINITY;       // pads the last group of four; never ranks ahead
     __syncthreads();
   } else {
     __syncthreads();
@@ -485,24 +483,21 @@ __global__ void __launch_bounds__(kSelThreads) rocket_select_kernel(const __half
   int base = 0;
   if (ns <= (int)blockDim.x) {
     // few pages: each thread ranks its page by counting the pages ahead of it under
-    // (score desc, page asc)
+    // (score desc, page asc).  The scores' order-preserving keys are counted: with a NaN among the scores (infinite
+    // keys) a comparison of values would give several pages one rank and list more than k.
     const int i = threadIdx.x;
     int flag = 0;
+    uint32_t* keys = reinterpret_cast<uint32_t*>(ssc);
+    if (i < ((ns + 3) & ~3)) keys[i] = i < ns ? f32_key(ssc[i]) : 0u;   // (its own score; pads never rank ahead)
+    __syncthreads();
     if (i < ns && k > 0) {
-      const float si = ssc[i];
+      const uint32_t own = keys[i];
       int rank = 0;
-      if (fast) {                         // scores padded to a multiple of four with -inf
 #pragma unroll 4
-        for (int j = 0; j < ns; j += 4) {
-          const float4 v = *reinterpret_cast<const float4*>(ssc + j);
-          rank += (v.x > si || (v.x == si && j < i)) + (v.y > si || (v.y == si && j + 1 < i)) +
-                  (v.z > si || (v.z == si && j + 2 < i)) + (v.w > si || (v.w == si && j + 3 < i));
-        }
-      } else {
-        for (int j = 0; j < ns; ++j) {
-          const float sj = ssc[j];
-          rank += (sj > si || (sj == si && j < i)) ? 1 : 0;
-        }
+      for (int j = 0; j < ns; j += 4) {
+        const uint4 v = *reinterpret_cast<const uint4*>(keys + j);
+        rank += (v.x > own || (v.x == own && j < i)) + (v.y > own || (v.y == own && j + 1 < i)) +
+                (v.z > own || (v.z == own && j + 2 < i)) + (v.w > own || (v.w == own && j + 3 < i));
       }
       flag = rank < k;
     }

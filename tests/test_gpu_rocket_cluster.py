@@ -134,3 +134,47 @@ def test_longest_accepted_cache(B, Hkv, D, dims):
         assert_close(out.float().cpu(), ref.float().cpu(), f"step {s}")
         for name in a.t:
             assert torch.equal(a.t[name], c.t[name]), (s, name)
+
+
+@pytest.mark.parametrize("n,pages", [(1600, 9), (4160, 64), (16400, 200), (32000, 30)])
+@pytest.mark.parametrize("D,dims", [(64, 16), (128, 32)])
+def test_nan_and_infinite_values_choose_real_pages(D, dims, n, pages):
+    """A query with NaNs or infinite cached keys in one batch entry: its page list still holds distinct pages in range and
+    nothing is written behind it, and the other entry is not touched."""
+    torch = torch_cuda()
+    dev = torch.device("cuda")
+    g = torch.Generator(device=dev).manual_seed(n)
+    B, Hkv, G = 4, 2, 4
+    cap = (n + 31) // 16 * 16
+    cfg = mkv.config(mkv.MKV_ROCKET, B, Hkv * G, Hkv, D, snap_window=1, snap_keep=cap, topk_pages=pages, topq_dims=dims)
+    c = caches.alloc_cache(cfg, cap, device=dev)
+    for x in ("k", "v"):
+        c.t[x].normal_(generator=g)
+    c.t["k"][1, :, ::37, ::3] = float("inf")
+    c.t["k"][1, :, 5::61, 1::3] = float("-inf")
+    pg = c.t["k"].unflatten(2, (cap // 16, 16))
+    c.t["kmin"].copy_(pg.amin(3).transpose(2, 3))
+    c.t["kmax"].copy_(pg.amax(3).transpose(2, 3))
+    c.t["T_len"].fill_(n)
+    clean = torch.randn((B, Hkv * G, D), generator=g, device=dev).half()
+    q = clean.clone()
+    q[1, :, ::2] = q[1, :, ::2].clamp(min=0)           # (0 * inf)
+    q[2, 1, ::5] = float("nan")
+    q[3] = float("nan")
+    ns = (n - 1) // 16
+    for call in ("select", "fused"):
+        lists = {}
+        for name, x in (("clean", clean), ("q", q)):
+            buf = torch.full((B * Hkv * pages + 64,), -77, dtype=torch.int32, device=dev)
+            out = torch.empty_like(q)
+            if call == "select":
+                mkv.mkv_rocket_select(cfg, x.data_ptr(), c.c, buf.data_ptr())
+            else:
+                mkv.mkv_rocket_decode(cfg, x.data_ptr(), c.c, buf.data_ptr(), out.data_ptr())
+                assert not bool(out[0].isnan().any())
+            assert mkv.mkv_get_status() == 0
+            assert bool((buf[B * Hkv * pages:] == -77).all())
+            lists[name] = buf[:B * Hkv * pages].view(B, Hkv, pages)
+        x = lists["q"]
+        assert torch.equal(x[0], lists["clean"][0])
+        assert bool((x >= 0).all() and (x < ns).all() and (x[..., 1:] > x[..., :-1]).all())
