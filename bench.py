@@ -782,6 +782,25 @@ def oracle_tokens_per_s_all_cores(name: str, w, budget_s: float, seed: int = 0):
 
 # --------------------------------------------------------------------------- main
 
+def short_line(line: dict) -> dict:
+    """The printed line: the headline as it is, of every other workload its rate alone (tokens/s; per_config also the
+    decode launch's share of the measured copy bandwidth) and of the prefill-side calls their time.  A reader that
+    keeps only the last few thousand characters of the output still has the whole line; --details writes the full rows."""
+    out = dict(line)
+    if "per_config" in out:
+        out["per_config"] = {name: [round(row["tokens_per_s"], 1), round(row["frac_of_measured_peak"], 3)]
+                             for name, row in out["per_config"].items()}
+    if "sweep" in out:                           # "kvquant_nuq4_b32_t4096": under its batch and context
+        out["sweep"] = {}
+        for name, row in line["sweep"].items():
+            config, b, t = name.rsplit("_", 2)
+            out["sweep"].setdefault(f"{b}_{t}", {})[config] = round(row["tokens_per_s"])
+    if "setup" in out:
+        out["setup"] = {name: {"ms": round(row["ms"], 4), "frac": round(row["roofline"]["frac"], 3)}
+                        for name, row in out["setup"].items()}
+    return out
+
+
 def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("--gpus", type=int, default=1)
@@ -802,6 +821,7 @@ def main():
     ap.add_argument("--cpu-all-cores", type=int, default=1, help="1: also time the oracle on every host core")
     ap.add_argument("--setup", type=int, default=1,
                     help="1: also time the prefill-side calls (H2O prefill, SnapKV compression) on their workloads")
+    ap.add_argument("--details", default="", help="file for the full rows of every workload, as JSON")
     ap.add_argument("--only-setup", type=int, default=0,
                     help="profiling: time only the prefill-side calls and print their JSON (not a bench line)")
     ap.add_argument("--setup-batch", type=int, default=None,
@@ -937,7 +957,10 @@ def main():
                 line["cpu_baseline_all_cores"] = {
                     "value": va, "unit": "tokens/s", "cores": n, "kind": "oracle", "extrapolated": True,
                     "sample": f"{n} single-threaded worker processes (nproc = {n}), each as the one-core sample"}
-        print(json.dumps(line))
+        if args.details:
+            with open(args.details, "w") as f:
+                json.dump(line, f, indent=1)
+        print(json.dumps(short_line(line)))
     if world > 1:
         torch.distributed.destroy_process_group()
 

@@ -116,3 +116,24 @@ def test_reference_arm_prints_the_contract_line():
     assert cb["kind"] == "oracle" and cb["cores"] >= 1 and cb["value"] == line["value"] and cb["sample"]
     assert line["e2e"] == {"value": line["value"], "unit": line["unit"], "h2d_bytes_per_step": 0,
                            "d2h_bytes_per_step": 0}
+
+
+def test_the_printed_line_is_short():
+    """With every workload measured the line stays within what a reader of the output's last characters keeps, and the
+    headline's keys are untouched."""
+    import json
+    import bench
+    import synth
+    row = {"tokens_per_s": 123456.78901234567, "frac_of_measured_peak": 0.78901234567, "decode_launch_ms": 0.123456789012345,
+           "step_paths_ms": {"kvquant_step": 1.23456789012345}, "note": "x" * 90, "kv_bytes_peak": 41337356288}
+    names = [synth.sweep(m, lv, T, B).name for (T, B) in synth.SWEEP_POINTS for (m, lv) in synth.SWEEP_CONFIGS]
+    assert len(names) == 40
+    call = {"ms": 25.75859260559082, "roofline": {"frac": 0.7012345678901, "note": "y" * 90}}
+    head = {"metric": bench.METRIC, "value": 1.0, "config": {"workload": "w"}, "clocks": {"sm_mhz": 2070, "reasons": []}}
+    line = dict(head, per_config={f"config_{i}_b16_t16384": row for i in range(5)}, sweep={n: row for n in names},
+                setup={"h2o20": call, "rocket1024": call})
+    short = bench.short_line(line)
+    assert {k: short[k] for k in head} == head
+    assert sum(len(x) for x in short["sweep"].values()) == 40 and short["sweep"]["b32_t4096"]["kvquant_nuq4"] == 123457
+    assert short["setup"]["h2o20"] == {"ms": 25.7586, "frac": 0.701}
+    assert len(json.dumps(short)) < 2000 and line["sweep"][names[0]] is row
