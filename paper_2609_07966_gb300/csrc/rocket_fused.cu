@@ -393,6 +393,9 @@ __global__ void __launch_bounds__(kRfThreads, 2) rocket_fused_kernel(const RfArg
         }
       }
       if constexpr (CL > 1) {
+        // (waited for before the end: a CTA that does not wait for scores, since it found no candidate page or its
+        // bounded wait ran out, stays until the others have sent theirs)
+        asm volatile("barrier.cluster.arrive.relaxed.aligned;\n" ::: "memory");
         if (ns > 0) wait_received(&bar[0]);
       } else {
         __syncthreads();
@@ -746,6 +749,7 @@ __global__ void __launch_bounds__(kRfThreads, 2) rocket_fused_kernel(const RfArg
       }
     }
   }
+  if constexpr (CL > 1) asm volatile("barrier.cluster.wait.aligned;\n" ::: "memory");
   if (!append) return;
   // the appended token filled its page: the page's per-dim min and max (its other rows from the cache)
   if (tail_warp && room && n % kPage == 0) {
