@@ -71,7 +71,6 @@ constexpr uint64_t kWaitNs = 1000000000ull;   // a bounded wait gives up after 1
 // gains more from four accumulator buffers, which let the tensor core run further ahead of it.
 template <int TN>
 struct Tiling {
-  static constexpr int kTN = TN;
   static constexpr int kNB = 512 / TN;            // accumulator buffers: all 512 tensor-memory columns
   static constexpr int kS = TN == 256 ? 2 : 4;    // operand stages
   static constexpr bool kAll = TN == 256;         // all epilogue warps read each product (else: a group of them)

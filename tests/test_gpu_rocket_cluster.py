@@ -178,3 +178,38 @@ def test_nan_and_infinite_values_choose_real_pages(D, dims, n, pages):
         x = lists["q"]
         assert torch.equal(x[0], lists["clean"][0])
         assert bool((x >= 0).all() and (x < ns).all() and (x[..., 1:] > x[..., :-1]).all())
+
+
+# units whose clusters have 4, 2 and 1 CTAs
+@pytest.mark.parametrize("B,Hkv,G,D", [(4, 8, 4, 128), (7, 8, 1, 64), (14, 8, 2, 64), (10, 10, 4, 128), (16, 8, 4, 128), (33, 4, 8, 64)])
+def test_step_equals_append_then_decode_beyond_16_units(B, Hkv, G, D):
+    """mkv_rocket_step against mkv_append_kv + mkv_rocket_decode on twin caches, bit for bit: empty and one-page entries,
+    pages completed, caches that fill up."""
+    torch = torch_cuda()
+    dev = torch.device("cuda")
+    g = torch.Generator(device=dev).manual_seed(B * D)
+    T_cap, steps, pages = 112, 20, 3
+    cfg = mkv.config(mkv.MKV_ROCKET, B, Hkv * G, Hkv, D, snap_window=1, snap_keep=T_cap, topk_pages=pages, topq_dims=D // 4)
+    a, c = (caches.alloc_cache(cfg, T_cap, device=dev) for _ in range(2))
+    for x in ("k", "v"):
+        a.t[x].normal_(generator=g)
+    pg = a.t["k"].unflatten(2, (T_cap // 16, 16))
+    a.t["kmin"].copy_(pg.amin(3).transpose(2, 3))
+    a.t["kmax"].copy_(pg.amax(3).transpose(2, 3))
+    a.t["T_len"].copy_(torch.tensor([[0, 15, 16, 47, 60, 100, 112][b % 7] for b in range(B)], dtype=torch.int32))
+    for x in a.t:
+        c.t[x].copy_(a.t[x])
+    for s in range(steps):
+        q = torch.randn((B, Hkv * G, D), generator=g, device=dev).half()
+        kn, vn = (torch.randn((B, Hkv, D), generator=g, device=dev).half() for _ in range(2))
+        ia, ic = (torch.full((B, Hkv, pages), -7, dtype=torch.int32, device=dev) for _ in range(2))
+        oa, oc = torch.empty_like(q), torch.empty_like(q)
+        mkv.mkv_append_kv(cfg, kn.data_ptr(), vn.data_ptr(), a.c)
+        fa = mkv.mkv_get_status()
+        mkv.mkv_rocket_decode(cfg, q.data_ptr(), a.c, ia.data_ptr(), oa.data_ptr())
+        mkv.mkv_rocket_step(cfg, q.data_ptr(), kn.data_ptr(), vn.data_ptr(), c.c, ic.data_ptr(), oc.data_ptr())
+        assert mkv.mkv_get_status() == fa
+        assert torch.equal(oa, oc) and torch.equal(ia, ic), s
+        for x in a.t:
+            assert torch.equal(a.t[x], c.t[x]), (s, x)
+    assert fa == mkv.MKV_FLAG_CACHE_FULL if B >= 6 else fa == 0
