@@ -22,7 +22,11 @@ __host__ __device__ __forceinline__ int64_t ceil_div_dev(int64_t a, int64_t b) {
 // for that grid's completion and memory before its first global access, then lets its own
 // successor be scheduled (which waits the same way); a successor can only be scheduled once every
 // CTA of this grid has passed this point, so it never holds resources a CTA of this grid is waiting
-// for.  (The KVQuant and fused RocketKV kernels launch plainly: there it measured slower.)
+// for.  The two launches of mkv_kvquant_step have the attribute as well and place the two
+// instructions themselves: the quantization waits first and then lets the decode start, which reads
+// tables and the query (finished before the quantization was allowed to run) and waits before it touches
+// the cache; near its end the decode lets the next step's quantization be scheduled.  The KVQuant calls one by
+// one and the fused RocketKV step launch plainly: there the attribute measured slower.
 __device__ __forceinline__ void pdl_wait_and_trigger() {
   asm volatile("griddepcontrol.wait;\n" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
